@@ -43,7 +43,9 @@ extern "C" {
 
 /* Arithmetic of the dense contractions (separator Schur updates and selected-inverse
  * products).  Diagonal pivot blocks, their inverses and the residue sum are FP64 in both. */
-#define NDSI_PREC_FP64   0   /* FP64 operands and accumulation on the CUDA cores */
+#define NDSI_PREC_FP64   0   /* FP64 operands on the CUDA cores: products exact in 57-bit fixed point per
+                                operand row and 32 inner indices (integer multiply-adds), summed
+                                in FP64 */
 #define NDSI_PREC_SPLIT  1   /* FP64 emulated by BF16 slices on the tcgen05 tensor cores */
 
 typedef struct ndsi_plan ndsi_plan;
@@ -299,8 +301,8 @@ int ndsi_profile_enable(ndsi_plan* plan, int32_t enable);
  * the faster path per step for all later calls on the plan.  Both paths meet the split-mode
  * tolerance, so only speed changes.  Small steps (few tiles, short inner dimension) usually go
  * to the CUDA cores, separator-sized ones to the tensor cores.  A step whose tensor-core time is
- * below the least time the FP64 cores could need for it (its issued FP64 flops at the DFMA rate
- * measured on the device, as ndsi_fp64_peak) is decided without an FP64 run, so on large systems
+ * below the least time the CUDA cores could need for it (their integer multiply-add rate) is
+ * decided without an FP64 run, so on large systems
  * the FP64 sweeps time only the small steps.  A plan with the default accumulators (one per
  * slice scale) then times every tensor-core step once more with five accumulator bands (48
  * complex columns per tile instead of 40, within the same tolerance) and keeps the faster tile per
@@ -347,9 +349,9 @@ int ndsi_profile_read(const ndsi_plan* plan, ndsi_profile_entry* out, int32_t ma
 
 /* FP64 throughput of the current GPU in TFLOP/s (host *tflops_out): every SM runs 2048 threads
  * of eight independent fused multiply-add chains (2 flops each), timed with CUDA events on
- * `stream`, best of five launches after a warm-up (about 0.1 s in all).  This is the measured
- * ceiling of the FP64 path's kernels (the paper's arithmetic is FP64 throughout, Sec. II; GB300
- * runs FP64 on the CUDA cores only), against which their roofline fractions are quoted.
+ * `stream`, best of five launches after a warm-up (about 0.1 s in all).  The paper's arithmetic is
+ * FP64 throughout (Sec. II), which GB300 runs on the CUDA cores only, at 1/64 of its FP32 rate; the
+ * FP64 path's products run on the integer pipe instead and are not bound by this figure.
  * Synchronises `stream`.  Errors: NDSI_ERR_INVALID (NULL output), NDSI_ERR_CUDA. */
 int ndsi_fp64_peak(double* tflops_out, void* stream);
 

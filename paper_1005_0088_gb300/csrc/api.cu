@@ -100,7 +100,11 @@ int alloc_workspace(Workspace& W, const Plan& P, int32_t np) {
     W = Workspace{};
     W.front_stride = P.front_total;
     W.scr_stride = P.scr_total;
-    NDSI_CK(cudaMalloc(&W.fronts, sizeof(double2) * static_cast<size_t>(W.front_stride) * np));
+    const size_t front_bytes = sizeof(double2) * static_cast<size_t>(W.front_stride) * np;
+    NDSI_CK(cudaMalloc(&W.fronts, front_bytes + scale_bytes(P)));
+    W.scale_any = reinterpret_cast<int*>(reinterpret_cast<char*>(W.fronts) + front_bytes);
+    W.scale_f = reinterpret_cast<int16_t*>(W.scale_any + 64);
+    W.scale_pair = W.scale_f + P.n;
     NDSI_CK(cudaMalloc(&W.scr, sizeof(double2) * static_cast<size_t>(W.scr_stride) * np));
     W.np_cap = np;
     return NDSI_OK;
@@ -675,6 +679,8 @@ int ndsi_factor_poles(ndsi_plan* h, const double* H, const double* S, const doub
     }
     const double *Hd, *Sd;
     rc = device_inputs(h, H, S, &Hd, &Sd, st);
+    if (!rc && launch_basis_scale(h->P, h->T, Sd, f->W, st) != cudaSuccess)
+        rc = fail(NDSI_ERR_CUDA, "ndsi_factor_poles: basis scaling launch failed");
     if (!rc) rc = run_phase(h, f->W, f->SB, 0, Hd, Sd, f->zd, 0, n_poles, st);
     if (rc) {
         cleanup();
@@ -990,6 +996,7 @@ int sweep(ndsi_plan* h, const double* Hd, const double* Sd, int32_t nq, int32_t 
           const std::vector<int>& part_off, double* rho_d, double* ne_d, double* e_d, cudaStream_t st) {
     int rc;
     const int32_t ns = h->P.n_systems;
+    NDSI_CK(launch_basis_scale(h->P, h->T, Sd, h->W, st));
     for (int32_t q0 = 0; q0 < nq;) {
         const bool far = q0 >= n_near;
         const int32_t np = std::min(chunk, (far ? nq : n_near) - q0);
@@ -1150,13 +1157,14 @@ int ndsi_autotune(ndsi_plan* h, const double* H, const double* S, double mu, dou
     // with every eligible GEMM on the FP64 CUDA cores (each after an untimed warm-up sweep); each
     // launch then keeps the faster of the two.  Both choices meet the split tolerance, so the
     // result only changes speed.  The profiler's own counters are left as they were.
-    // A step whose tensor-core time is already below the least time the FP64 path could take
-    // (its issued FP64 flops, 3 of every 4 counted, at the measured DFMA rate) is decided without
-    // running it on the FP64 cores: only the other steps are timed there, so the FP64 passes cost
-    // about as much as tensor-core ones on large systems.
-    double peak = 0.0;
-    rc = fp64_rate(st, &peak);
-    if (rc) return rc;
+    // A step whose tensor-core time is already below the least time the FP64 path could take (twelve
+    // integer multiply-adds per complex product at 64 lanes per clock and SM, k_gemm_f64's bound) is
+    // decided without running it on the CUDA cores: only the other steps are timed there.
+    int dev = 0, sms = 0, khz = 0;
+    NDSI_CK(cudaGetDevice(&dev));
+    NDSI_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    NDSI_CK(cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev));
+    const double peak = 8.0 * 64.0 / 12.0 * sms * khz * 1e3;  // 8-flop complex products per second
     Profiler saved = h->prof;
     h->prof.pending.clear();
     h->prof.used = 0;
@@ -1172,7 +1180,7 @@ int ndsi_autotune(ndsi_plan* h, const double* H, const double* S, double mu, dou
     for (size_t li = 0; li < nl && !rc; ++li) {
         const Launch& l = h->P.launches[li];
         if (!split_eligible(l)) continue;
-        const double fp64_min_ms = 0.75 * l.flops * points / (peak * 1e12) * 1e3;
+        const double fp64_min_ms = l.flops * points / peak * 1e3;
         decided[li] = t_split[li] <= fp64_min_ms ? 1 : 0;
     }
     for (int pass = 0; pass < 2 && !rc; ++pass) {

@@ -19,6 +19,15 @@ int ensure_solve_tables(ndsi_plan* h) {
     return NDSI_OK;
 }
 
+// Row exponents the solves with W's factors need (NULL for a normalised basis, where all are 0).
+int solve_scale(const Workspace& W, const int16_t** f, cudaStream_t st) {
+    int any = 0;
+    NDSI_CK(cudaMemcpyAsync(&any, W.scale_any, sizeof(int), cudaMemcpyDeviceToHost, st));
+    NDSI_CK(cudaStreamSynchronize(st));
+    *f = any ? W.scale_f : nullptr;
+    return NDSI_OK;
+}
+
 // Uniform [-1, 1) numbers from a counter (splitmix64 finaliser) for the starting block.
 double counter_uniform(uint64_t seed, uint64_t i) {
     uint64_t x = seed + 0x9E3779B97F4A7C15ull * (i + 1);
@@ -57,7 +66,14 @@ int ndsi_factors_solve(ndsi_factors* f, int32_t pole, const double* Y, int32_t k
     const bool x_dev = is_device_ptr(X_out);
     double2* xd = x_dev ? reinterpret_cast<double2*>(X_out) : f->solve_buf + f->solve_cap;
     NDSI_CK(cudaMemcpyAsync(yw, Y, bytes, cudaMemcpyDefault, st));
-    NDSI_CK(launch_solve(h->P, h->ST, f->W.fronts + static_cast<int64_t>(pole) * f->W.front_stride, yw, xd, k, st));
+    if (f->scaled < 0) {  // the factors' own scaling, read once
+        const int16_t* sf = nullptr;
+        rc = solve_scale(f->W, &sf, st);
+        if (rc) return rc;
+        f->scaled = sf ? 1 : 0;
+    }
+    NDSI_CK(launch_solve(h->P, h->ST, f->W.fronts + static_cast<int64_t>(pole) * f->W.front_stride, yw, xd, k,
+                         f->scaled ? f->W.scale_f : nullptr, st));
     if (!x_dev) NDSI_CK(cudaMemcpyAsync(X_out, xd, bytes, cudaMemcpyDeviceToHost, st));
     NDSI_CK(cudaStreamSynchronize(st));
     return NDSI_OK;
@@ -89,7 +105,10 @@ int ndsi_eigenstates(ndsi_plan* h, const double* H, const double* S, double xi, 
     if (!h->point_z) NDSI_CK(cudaMalloc(&h->point_z, sizeof(double2)));
     const double2 z = make_double2(xi, eta);
     NDSI_CK(cudaMemcpyAsync(h->point_z, &z, sizeof(double2), cudaMemcpyHostToDevice, st));
+    NDSI_CK(launch_basis_scale(h->P, h->T, Sd, h->W, st));
     rc = run_phase(h, h->W, h->SB, 0, Hd, Sd, h->point_z, 1, 1, st);
+    const int16_t* sf = nullptr;
+    if (!rc) rc = solve_scale(h->W, &sf, st);
     if (rc) return rc;
     // buffers: complex right-hand sides and solutions, V = [Re B | Im B], H V, S V, the block C
     const int mmax = 2 * block;
@@ -126,13 +145,13 @@ int ndsi_eigenstates(ndsi_plan* h, const double* H, const double* S, double xi, 
         // (B2): b = (z S - H)^{-1} S c, the shift-invert product with the factors of z
         NDSI_CK(launch_spmm(h->T.rowptr, h->T.col, Sd, n, cb.as<double>(), m, vb.as<double>(), m, m, st));
         NDSI_CK(launch_real_to_complex(vb.as<double>(), n * m, yb.as<double2>(), st));
-        NDSI_CK(launch_solve(h->P, h->ST, h->W.fronts, yb.as<double2>(), xb.as<double2>(), m, st));
+        NDSI_CK(launch_solve(h->P, h->ST, h->W.fronts, yb.as<double2>(), xb.as<double2>(), m, sf, st));
         for (int r = 0; r < refine; ++r) {
             // iterative refinement in FP64: x += (zS - H)^{-1} (y - (zS - H) x)
             NDSI_CK(launch_real_to_complex(vb.as<double>(), n * m, yb.as<double2>(), st));
             NDSI_CK(launch_shifted_residual(h->T.rowptr, h->T.col, Hd, Sd, n, z, xb.as<double2>(), yb.as<double2>(),
                                             rb.as<double2>(), m, st));
-            NDSI_CK(launch_solve(h->P, h->ST, h->W.fronts, rb.as<double2>(), yb.as<double2>(), m, st));
+            NDSI_CK(launch_solve(h->P, h->ST, h->W.fronts, rb.as<double2>(), yb.as<double2>(), m, sf, st));
             NDSI_CK(launch_complex_add(xb.as<double2>(), yb.as<double2>(), n * m, st));
         }
         // (B3) in the real span of Re b and Im b

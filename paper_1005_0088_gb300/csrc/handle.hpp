@@ -115,6 +115,7 @@ struct ndsi_factors {
     ndsi::SplitBuffers SB;
     double2* zd = nullptr;
     int32_t np = 0;
+    int8_t scaled = -1;     // the basis scaling of these factors is not trivial (-1: not read yet)
     bool inverted = false;  // ndsi_selinv has replaced the factors by G
     int64_t split_gen = 0;  // split schedule generation the factors were made with
     double2* solve_buf = nullptr;  // work space of ndsi_factors_solve (two n x k blocks)

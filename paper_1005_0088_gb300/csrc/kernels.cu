@@ -18,6 +18,11 @@ namespace {
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
+// x 2^e (e = 0 for every entry of a normalised basis).
+__device__ __forceinline__ double scale2(double x, int e) {
+    if (e == 0) return x;
+    return e >= -1022 && e <= 1023 ? x * __hiloint2double((1023 + e) << 20, 0) : ldexp(x, e);
+}
 __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 
 // ---------------------------------------------------------------------------------------------
@@ -65,7 +70,38 @@ __global__ void __launch_bounds__(256) k_assemble(const NodeDev* __restrict__ no
     }
 }
 
-// X = z S - H on the level's entries (each front element receives at most one entry).
+// Exponents of the basis scaling (launch_basis_scale): f_i from the exponent of S_ii, one thread per
+// basis function; S_ii <= 0 or non-finite leaves f_i = 0.
+__global__ void __launch_bounds__(256) k_basis_scale(const int64_t* __restrict__ rowptr,
+                                                     const int32_t* __restrict__ col, int64_t n,
+                                                     const double* __restrict__ S, int16_t* __restrict__ f,
+                                                     int* __restrict__ any) {
+    const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    int v = 0;
+    if (i < n) {
+        int64_t lo = rowptr[i], hi = rowptr[i + 1] - 1;
+        while (lo < hi) {
+            const int64_t mid = (lo + hi) >> 1;
+            if (col[mid] < i) lo = mid + 1;
+            else hi = mid;
+        }
+        const int b = col[lo] == i ? __double2hiint(S[lo]) >> 20 : 0;  // sign and exponent field
+        if (b > 0 && b < 0x7FF) v = -((b - 1022) >> 1);
+        f[i] = static_cast<int16_t>(v);
+    }
+    if (__syncthreads_or(v != 0) && threadIdx.x == 0) *any = 1;
+}
+__global__ void __launch_bounds__(256) k_pair_scale(const int64_t* __restrict__ rowptr,
+                                                    const int32_t* __restrict__ col, int64_t n,
+                                                    const int16_t* __restrict__ f, int16_t* __restrict__ pair) {
+    const int64_t i = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
+    if (i >= n) return;
+    const int fi = f[i];
+    for (int64_t k = rowptr[i] + (threadIdx.x & 31); k < rowptr[i + 1]; k += 32) pair[k] = static_cast<int16_t>(fi + f[col[k]]);
+}
+
+// X = z S - H on the level's entries (each front element receives at most one entry), scaled by the
+// entry's pair exponent.
 // z[sys * zstride + pole] is the point of the entry's system (systems of a batch have their own
 // mu and kT).
 __global__ void __launch_bounds__(256) k_scatter(const int64_t* __restrict__ idx, int64_t first,
@@ -73,6 +109,7 @@ __global__ void __launch_bounds__(256) k_scatter(const int64_t* __restrict__ idx
                                                  const int32_t* __restrict__ entry_sys,
                                                  const double* __restrict__ H,
                                                  const double* __restrict__ S,
+                                                 const int16_t* __restrict__ pair,
                                                  const double2* __restrict__ z, int64_t zstride,
                                                  double2* __restrict__ F, int64_t stride) {
     double2* Fp = F + static_cast<int64_t>(blockIdx.y) * stride;
@@ -83,8 +120,9 @@ __global__ void __launch_bounds__(256) k_scatter(const int64_t* __restrict__ idx
         const double2 zq = z[entry_sys[k] * zstride + blockIdx.y];
         const double h = H[k], s = S[k];
         double2 v = Fp[off];
-        v.x += zq.x * s - h;
-        v.y += zq.y * s;
+        const int pe = pair[k];
+        v.x += scale2(zq.x * s - h, pe);
+        v.y += scale2(zq.y * s, pe);
         Fp[off] = v;
     }
 }
@@ -237,123 +275,221 @@ __global__ void __launch_bounds__(32) k_diaginv_sweep(const DiagItem* __restrict
 }
 
 // ---------------------------------------------------------------------------------------------
-// Batched complex FP64 GEMM on the CUDA cores: C = alpha op(A) op(B) + beta C for every tile of
-// a schedule step.  TILE x TILE output tile (32, or 16 for launches of small items, where a 32
-// tile would spend its multiply-adds on padding), K step 16, 64 threads with (TILE/8)^2 outputs
-// each.  The complex product uses three real products per element (Re = P1 - P2,
-// Im = P3 - P1 - P2 with P1 = Ar Br, P2 = Ai Bi, P3 = (Ar + Ai)(Br + Bi)): GB300's FP64 rate is
-// the bound here, and the third real product saves a quarter of the DFMAs.
-constexpr int BK = 16;
+// Fixed-point products.  GB300 issues one warp-wide FP64 instruction per SM every 16-19 clocks (1.7-2
+// lanes a clock; 64 clocks per sub-partition) but 59 lanes a clock of 32 x 32 + 64-bit integer
+// multiply-adds (both measured), so products of complex matrices are formed in 57-bit fixed point:
+// over at most 32 inner indices every row of op(A) and column of op(B) is scaled by a power of two
+// and cut to x = (h 2^29 + l) 2^(E - 57), |h| <= 2^28, -2^28 <= l < 2^28.  Twelve integer
+// multiply-adds per complex product accumulate the h h and h l + l h sums exactly in 64 bits
+// (|sum| <= 2^62 and 2^63 over 32 terms; l l, below 2^-57 of the row times column maximum, is
+// dropped), and the sum is rounded once to FP64.  The error of an output is about 2^-57 of (row
+// maximum) x (column maximum) per term plus that one rounding, against one FP64 rounding per term
+// and accumulator of a DFMA loop.  The basis functions are brought to a common scale beforehand
+// (launch_basis_scale), so that a row's maximum speaks for the row.
+// Rows or columns holding an infinity or NaN give NaN.
+constexpr int kFixK = 32;          // inner indices per exact integer sum
+constexpr int kFixNonFinite = 1 << 20;  // row exponent of a row holding an infinity or NaN
 
-template <int OP>
-__device__ __forceinline__ double2 load_op(const double2* __restrict__ X, int ld, int r, int c) {
-    if (OP == OP_N) return X[r + static_cast<int64_t>(c) * ld];
-    if (OP == OP_T) return X[c + static_cast<int64_t>(r) * ld];
-    const int hi = r > c ? r : c, lo = r > c ? c : r;
-    return X[hi + static_cast<int64_t>(lo) * ld];
+// Digits of x at row exponent field `emax` (x == 0 or its exponent field <= emax): F = x 2^(57 - E) cut
+// towards zero.
+__device__ __forceinline__ void fix_digits(double x, int emax, int& h, int& l) {
+    const int64_t b = __double_as_longlong(x);
+    const int ex = static_cast<int>((b >> 52) & 0x7FF);
+    const uint64_t m = (static_cast<uint64_t>(b) << 10 & 0x3FFFFFFFFFFFFFFFull) | 0x4000000000000000ull;  // 1.f at bit 62
+    const int sh = ex ? min(6 + emax - ex, 63) : 63;
+    int64_t f = static_cast<int64_t>(m >> sh);
+    f = b < 0 ? -f : f;
+    l = static_cast<int>(static_cast<uint32_t>(f) << 3) >> 3;
+    h = static_cast<int>((f - l) >> 29);
 }
 
-template <int OPA, int OPB, int TILE>
-__global__ void __launch_bounds__(64) k_gemm_f64(const GemmItem* __restrict__ items,
-                                                 const GemmTile* __restrict__ tiles, int64_t tfirst,
-                                                 int64_t ifirst, const double2* __restrict__ Abuf,
-                                                 int64_t sA, const double2* __restrict__ Bbuf,
-                                                 int64_t sB, double2* __restrict__ Cbuf, int64_t sC,
-                                                 double alpha, double beta, int lower) {
-    constexpr int MT = TILE / 8;           // outputs per thread along each edge
-    constexpr int LD = TILE * BK / 64;     // operand elements each thread stages per K step
-    __shared__ double As[3][BK][TILE + 1];
-    __shared__ double Bs[3][BK][TILE + 1];
+__device__ __noinline__ double fix_to_double_slow(int64_t t, uint32_t rem, int e) {
+    if (e >= kFixNonFinite / 2) return __longlong_as_double(0x7FF8000000000000ll);
+    return ldexp(ldexp(static_cast<double>(t), 29) + static_cast<double>(rem), e + 29);
+}
+// (hh 2^58 + mid 2^29) 2^e rounded to FP64, with integer operations.
+__device__ __forceinline__ double fix_to_double(int64_t hh, int64_t mid, int e) {
+    const int64_t t = hh + (mid >> 29);
+    const uint32_t rem = static_cast<uint32_t>(mid) & 0x1FFFFFFFu;
+    const bool neg = t < 0;
+    const uint64_t tm = static_cast<uint64_t>(neg ? (rem ? ~t : -t) : t);
+    const uint32_t rm = neg ? (0x20000000u - rem) & 0x1FFFFFFFu : rem;
+    const int s = min(__clzll(static_cast<long long>(tm)), 29);
+    uint64_t u = (tm << s) | (rm >> (29 - s));
+    const int lz = __clzll(static_cast<long long>(u));
+    const int biased = 63 - lz + 58 - s + e + 1023;
+    if (biased <= 0 || biased >= 2046) return u || e >= kFixNonFinite / 2 ? fix_to_double_slow(t, rem, e) : 0.0;
+    u <<= lz & 63;
+    const uint64_t mant = (u >> 11) + ((u >> 10) & 1);  // in [2^52, 2^53]; zero when u is
+    const uint64_t bits = u ? (static_cast<uint64_t>(biased - 1) << 52) + mant : 0;
+    return __longlong_as_double(static_cast<int64_t>(bits | static_cast<uint64_t>(neg) << 63));
+}
+
+
+// One complex product into the four exact sums: (a.x + i a.z) (b.x + i b.z) with low digits y, w.
+struct FixSum {
+    int64_t rh, rm, ih, im;
+};
+__device__ __forceinline__ void fix_mac(FixSum& c, const int4& a, const int4& b) {
+    const int nzh = -a.z, nzl = -a.w;
+    c.rh += static_cast<int64_t>(a.x) * b.x;
+    c.rm += static_cast<int64_t>(a.x) * b.y;
+    c.ih += static_cast<int64_t>(a.x) * b.z;
+    c.im += static_cast<int64_t>(a.x) * b.w;
+    c.rm += static_cast<int64_t>(a.y) * b.x;
+    c.im += static_cast<int64_t>(a.y) * b.z;
+    c.ih += static_cast<int64_t>(a.z) * b.x;
+    c.im += static_cast<int64_t>(a.z) * b.y;
+    c.rh += static_cast<int64_t>(nzh) * b.z;
+    c.rm += static_cast<int64_t>(nzh) * b.w;
+    c.im += static_cast<int64_t>(a.w) * b.x;
+    c.rm += static_cast<int64_t>(nzl) * b.z;
+}
+__device__ __forceinline__ double2 fix_value(const FixSum& c, int e) {
+    return make_double2(fix_to_double(c.rh, c.rm, e), fix_to_double(c.ih, c.im, e));
+}
+__device__ __forceinline__ int expo_bits(double2 v) {
+    return max(__double2hiint(v.x) & 0x7FF00000, __double2hiint(v.y) & 0x7FF00000);
+}
+__device__ __forceinline__ int4 fix_digits2(double2 v, int emax) {
+    int4 q;
+    fix_digits(v.x, emax, q.x, q.y);
+    fix_digits(v.y, emax, q.z, q.w);
+    return q;
+}
+// Exponent a row's digits are stored with, from its largest exponent field.
+__device__ __forceinline__ int fix_expo(int emax) { return emax == 0x7FF ? kFixNonFinite : emax - 1022 - 57; }
+
+// ---------------------------------------------------------------------------------------------
+// Batched complex FP64 GEMM on the CUDA cores: C = alpha op(A) op(B) + beta C for every tile of
+// a schedule step, products in fixed point (above) over chunks of 32 inner indices, the chunks
+// added in FP64.  One CTA of 128 threads per 32 x 32 output tile, outputs 8 rows and 16 columns apart,
+// so that a ragged tile skips its empty 8-row and (per warp) 4-column groups and a tile on the
+// diagonal of a lower-triangle result those above it; operands are staged by cp.async and turned
+// into digits in place, two threads per operand row.  Four CTAs per SM overlap one CTA's loads and
+// conversion with the others' products.
+template <int OP>
+__device__ __forceinline__ int64_t op_offset(int ld, int r, int c) {
+    if (OP == OP_N) return r + static_cast<int64_t>(c) * ld;
+    if (OP == OP_T) return c + static_cast<int64_t>(r) * ld;
+    const int hi = r > c ? r : c, lo = r > c ? c : r;
+    return hi + static_cast<int64_t>(lo) * ld;
+}
+
+constexpr int kFixThreads = 128;
+// kc inner products of a thread's mi x nj outputs (FULL: 4 x 2); group (i, j) is skipped when all of it
+// lies above the diagonal, 8 i < d + 16 j (d <= -16: no group).
+template <bool FULL>
+__device__ __forceinline__ void fix_products(const int4 (*As)[kGemmTile + 1], const int4 (*Bs)[kGemmTile + 1], int kc,
+                                             int tx, int ty, int mi, int nj, int d, FixSum (&c)[4][2]) {
+#pragma unroll 1
+    for (int k = 0; k < kc; ++k) {
+        int4 b[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+            if (FULL || j < nj) b[j] = Bs[k][ty + 16 * j];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (!FULL && i >= mi) continue;
+            const int4 a = As[k][tx + 8 * i];  // re h, re l, im h, im l
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                if (!FULL && (j >= nj || 8 * i < d + 16 * j)) continue;
+                fix_mac(c[i][j], a, b[j]);
+            }
+        }
+    }
+}
+
+template <int OPA, int OPB>
+__global__ void __launch_bounds__(kFixThreads, 4)
+    k_gemm_f64(const GemmItem* __restrict__ items, const GemmTile* __restrict__ tiles, int64_t tfirst, int64_t ifirst,
+               const double2* __restrict__ Abuf, int64_t sA, const double2* __restrict__ Bbuf, int64_t sB,
+               double2* __restrict__ Cbuf, int64_t sC, double alpha, double beta, int lower) {
+    __shared__ int4 sh[2][kFixK][kGemmTile + 1];  // op(A) rows, op(B) columns: raw FP64, then digits
+    __shared__ int ex[2][kGemmTile];
     const GemmTile t = tiles[tfirst + blockIdx.x];
     const GemmItem it = items[ifirst + t.item];
     const int64_t pole = blockIdx.y;
     const double2* A = Abuf + pole * sA + it.a_off;
     const double2* B = Bbuf + pole * sB + it.b_off;
     double2* C = Cbuf + pole * sC + it.c_off;
-    const int tid = threadIdx.x;
-    const int tx = tid % 8, ty = tid / 8;
-    double p1[MT][MT], p2[MT][MT], p3[MT][MT];
+    // outputs (tx + 8 i, ty + 16 j); a warp holds 8 rows x 4 columns of each group
+    const int tid = threadIdx.x, tx = tid % 8, ty = tid / 8;
+    const int mrem = min(kGemmTile, it.M - t.m0), nrem = min(kGemmTile, it.N - t.n0);
+    const int mi = (mrem + 7) / 8;
+    const int nj = (nrem - (ty & ~3) + 15) / 16;  // column groups of this warp with a live column
+    // first row group of column group j that reaches the diagonal: 8 i + 7 >= n0 + (ty & ~3) + 16 j - m0
+    const int d = lower ? t.n0 - t.m0 + (ty & ~3) - 7 : -64;
+    double2 acc[4][2];
 #pragma unroll
-    for (int i = 0; i < MT; ++i)
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < MT; ++j) p1[i][j] = p2[i][j] = p3[i][j] = 0.0;
-    for (int k0 = 0; k0 < it.K; k0 += BK) {
-#pragma unroll
-        for (int u = 0; u < LD; ++u) {
-            const int e = tid + 64 * u;
-            int lm, lk;
-            if (OPA == OP_T) {
-                lk = e % BK;
-                lm = e / BK;
-            } else {
-                lm = e % TILE;
-                lk = e / TILE;
-            }
-            const int m = t.m0 + lm, k = k0 + lk;
-            const double2 v = (m < it.M && k < it.K) ? load_op<OPA>(A, it.lda, m, k) : make_double2(0.0, 0.0);
-            As[0][lk][lm] = v.x;
-            As[1][lk][lm] = v.y;
-            As[2][lk][lm] = v.x + v.y;
+        for (int j = 0; j < 2; ++j) acc[i][j] = make_double2(0.0, 0.0);
+    for (int k0 = 0; k0 < it.K; k0 += kFixK) {
+        const int kc = min(kFixK, it.K - k0);
+        auto stage = [&](int4* dst, const double2* src, bool ok) {
+            const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(ok ? 16 : 0) : "memory");
+        };
+#pragma unroll 4
+        for (int u = 0; u < kGemmTile * kFixK / kFixThreads; ++u) {
+            const int e = tid + u * kFixThreads;
+            const int f = e % 32, g = e / 32;
+            const int m = OPA == OP_T ? g : f, ka = OPA == OP_T ? f : g;
+            if (ka < kc) stage(&sh[0][ka][m], A + (m < mrem ? op_offset<OPA>(it.lda, t.m0 + m, k0 + ka) : 0), m < mrem);
+            const int n = OPB == OP_T ? f : g, kb = OPB == OP_T ? g : f;
+            if (kb < kc) stage(&sh[1][kb][n], B + (n < nrem ? op_offset<OPB>(it.ldb, k0 + kb, t.n0 + n) : 0), n < nrem);
         }
-#pragma unroll
-        for (int u = 0; u < LD; ++u) {
-            const int e = tid + 64 * u;
-            int ln, lk;
-            if (OPB == OP_T) {
-                ln = e % TILE;
-                lk = e / TILE;
-            } else {
-                lk = e % BK;
-                ln = e / BK;
-            }
-            const int n = t.n0 + ln, k = k0 + lk;
-            const double2 v = (n < it.N && k < it.K) ? load_op<OPB>(B, it.ldb, k, n) : make_double2(0.0, 0.0);
-            Bs[0][lk][ln] = v.x;
-            Bs[1][lk][ln] = v.y;
-            Bs[2][lk][ln] = v.x + v.y;
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
+        __syncthreads();
+        {
+            // two threads per operand row (even and odd inner indices): the largest exponent field
+            // of the chunk, then the digits in place
+            int4 (*x)[kGemmTile + 1] = sh[tid / 64];
+            const int row = (tid / 32 % 2) * 16 + tid % 16, kh = tid / 16 % 2;
+            int emax = 0;
+            for (int k = kh; k < kc; k += 2)
+                emax = max(emax, max(x[k][row].y & 0x7FF00000, x[k][row].w & 0x7FF00000));
+            emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 16)) >> 20;
+            for (int k = kh; k < kc; k += 2)
+                x[k][row] = fix_digits2(*reinterpret_cast<const double2*>(&x[k][row]), emax);
+            if (kh == 0) ex[tid / 64][row] = fix_expo(emax);
         }
         __syncthreads();
-#pragma unroll 2
-        for (int kk = 0; kk < BK; ++kk) {
-            double ar[MT], ai[MT], as[MT], br[MT], bi[MT], bs[MT];
+        if (nj > 0) {
+            FixSum c[4][2] = {};
+            if (mi == 4 && nj == 2 && d <= -16) fix_products<true>(sh[0], sh[1], kc, tx, ty, mi, nj, d, c);
+            else fix_products<false>(sh[0], sh[1], kc, tx, ty, mi, nj, d, c);
 #pragma unroll
-            for (int i = 0; i < MT; ++i) {
-                ar[i] = As[0][kk][tx + 8 * i];
-                ai[i] = As[1][kk][tx + 8 * i];
-                as[i] = As[2][kk][tx + 8 * i];
-            }
+            for (int i = 0; i < 4; ++i) {
+                if (i >= mi) continue;
+                const int ea = ex[0][tx + 8 * i];
 #pragma unroll
-            for (int j = 0; j < MT; ++j) {
-                br[j] = Bs[0][kk][ty + 8 * j];
-                bi[j] = Bs[1][kk][ty + 8 * j];
-                bs[j] = Bs[2][kk][ty + 8 * j];
-            }
-#pragma unroll
-            for (int i = 0; i < MT; ++i)
-#pragma unroll
-                for (int j = 0; j < MT; ++j) {
-                    p1[i][j] = fma(ar[i], br[j], p1[i][j]);
-                    p2[i][j] = fma(ai[i], bi[j], p2[i][j]);
-                    p3[i][j] = fma(as[i], bs[j], p3[i][j]);
+                for (int j = 0; j < 2; ++j) {
+                    if (j >= nj || 8 * i < d + 16 * j) continue;
+                    const double2 v = fix_value(c[i][j], ea + ex[1][ty + 16 * j]);
+                    acc[i][j] = k0 == 0 ? v : cadd(acc[i][j], v);
                 }
+            }
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int j = 0; j < MT; ++j) {
-        const int n = t.n0 + ty + 8 * j;
+    for (int j = 0; j < 2; ++j) {
+        const int n = t.n0 + ty + 16 * j;
 #pragma unroll
-        for (int i = 0; i < MT; ++i) {
+        for (int i = 0; i < 4; ++i) {
             const int m = t.m0 + tx + 8 * i;
             if (m < it.M && n < it.N && (!lower || m >= n)) {
                 double2* c = C + m + static_cast<int64_t>(n) * it.ldc;
-                const double re = p1[i][j] - p2[i][j];
-                const double im = p3[i][j] - p1[i][j] - p2[i][j];
-                double2 v = make_double2(alpha * re, alpha * im);
+                double2 v = acc[i][j];
+                if (alpha == -1.0) v = make_double2(-v.x, -v.y);
+                else if (alpha != 1.0) v = make_double2(alpha * v.x, alpha * v.y);
                 if (beta != 0.0) {
                     const double2 old = *c;
-                    v.x += beta * old.x;
-                    v.y += beta * old.y;
+                    if (beta == 1.0) v = cadd(v, old);
+                    else v = make_double2(fma(beta, old.x, v.x), fma(beta, old.y, v.y));
                 }
                 *c = v;
             }
@@ -409,6 +545,7 @@ __global__ void __launch_bounds__(256) k_gather(const NodeDev* __restrict__ node
 constexpr int kAccThreads = 256;
 
 __global__ void __launch_bounds__(kAccThreads) k_accumulate(const int64_t* __restrict__ out_map,
+                                                            const int16_t* __restrict__ pair,
                                                             int64_t k0, int64_t nnz,
                                                             const double2* __restrict__ F,
                                                             int64_t stride, int np,
@@ -422,12 +559,14 @@ __global__ void __launch_bounds__(kAccThreads) k_accumulate(const int64_t* __res
     double tr = 0.0;
     if (k < k0 + nnz) {
         const int64_t off = out_map[k];
-        double sum = accumulate ? rho[k] : 0.0;
+        const int pe = pair[k];
+        double sum = accumulate ? scale2(rho[k], -pe) : 0.0;
         for (int q = 0; q < np; ++q) {
             const double2 g = F[static_cast<int64_t>(q) * stride + off];
             const double2 w = c[q];
             sum += w.x * g.x - w.y * g.y;
         }
+        sum = scale2(sum, pe);
         rho[k] = sum;
         tr = sum * S[k];
     }
@@ -462,14 +601,18 @@ __global__ void __launch_bounds__(1024) k_reduce(const double* __restrict__ part
 }
 
 __global__ void __launch_bounds__(256) k_gather_pattern(const int64_t* __restrict__ out_map,
+                                                        const int16_t* __restrict__ pair,
                                                         int64_t nnz,
                                                         const double2* __restrict__ F,
                                                         int64_t stride, double2* __restrict__ G,
                                                         int64_t q0) {
     const int64_t q = blockIdx.y;
     for (int64_t k = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; k < nnz;
-         k += static_cast<int64_t>(gridDim.x) * blockDim.x)
-        G[(q0 + q) * nnz + k] = F[q * stride + out_map[k]];
+         k += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        const double2 g = F[q * stride + out_map[k]];
+        const int pe = pair[k];
+        G[(q0 + q) * nnz + k] = make_double2(scale2(g.x, pe), scale2(g.y, pe));
+    }
 }
 
 template <int OPA, int OPB>
@@ -478,14 +621,9 @@ cudaError_t gemm_launch(const Plan& P, const DevTables& T, const Launch& l, cons
     const double2* bufs[2] = {W.fronts, W.scr};
     const int64_t strides[2] = {W.front_stride, W.scr_stride};
     dim3 grid(static_cast<unsigned>(l.tcount), static_cast<unsigned>(np));
-    if (l.tile == kGemmTileSmall)
-        k_gemm_f64<OPA, OPB, kGemmTileSmall><<<grid, 64, 0, st>>>(
-            T.gemm_items, T.gemm_tiles, l.tfirst, l.first, bufs[l.bufA], strides[l.bufA], bufs[l.bufB],
-            strides[l.bufB], const_cast<double2*>(bufs[l.bufC]), strides[l.bufC], l.alpha, l.beta, l.lower);
-    else
-        k_gemm_f64<OPA, OPB, kGemmTile><<<grid, 64, 0, st>>>(
-            T.gemm_items, T.gemm_tiles, l.tfirst, l.first, bufs[l.bufA], strides[l.bufA], bufs[l.bufB],
-            strides[l.bufB], const_cast<double2*>(bufs[l.bufC]), strides[l.bufC], l.alpha, l.beta, l.lower);
+    k_gemm_f64<OPA, OPB><<<grid, kFixThreads, 0, st>>>(
+        T.gemm_items, T.gemm_tiles, l.tfirst, l.first, bufs[l.bufA], strides[l.bufA], bufs[l.bufB],
+        strides[l.bufB], const_cast<double2*>(bufs[l.bufC]), strides[l.bufC], l.alpha, l.beta, l.lower);
     (void)P;
     return cudaGetLastError();
 }
@@ -505,8 +643,8 @@ cudaError_t launch_step(const Plan& P, const DevTables& T, const Launch& l, cons
         case L_SCATTER: {
             const int64_t blocks = (l.count + 255) / 256;
             dim3 grid(static_cast<unsigned>(blocks < 4096 ? blocks : 4096), static_cast<unsigned>(np));
-            k_scatter<<<grid, 256, 0, st>>>(T.scatter_idx, l.first, l.count, T.asm_map, T.entry_sys, H, S, z,
-                                            zstride, W.fronts, W.front_stride);
+            k_scatter<<<grid, 256, 0, st>>>(T.scatter_idx, l.first, l.count, T.asm_map, T.entry_sys, H, S,
+                                            W.scale_pair, z, zstride, W.fronts, W.front_stride);
             return cudaGetLastError();
         }
         case L_DIAGINV: {
@@ -550,6 +688,14 @@ cudaError_t launch_step(const Plan& P, const DevTables& T, const Launch& l, cons
     }
 }
 
+cudaError_t launch_basis_scale(const Plan& P, const DevTables& T, const double* S, const Workspace& W, cudaStream_t st) {
+    cudaError_t e = cudaMemsetAsync(W.scale_any, 0, sizeof(int), st);
+    if (e != cudaSuccess) return e;
+    k_basis_scale<<<static_cast<unsigned>((P.n + 255) / 256), 256, 0, st>>>(T.rowptr, T.col, P.n, S, W.scale_f, W.scale_any);
+    k_pair_scale<<<static_cast<unsigned>((P.n + 7) / 8), 256, 0, st>>>(T.rowptr, T.col, P.n, W.scale_f, W.scale_pair);
+    return cudaGetLastError();
+}
+
 cudaError_t kernels_init() {
     const int sm64 = 64 * 65 * static_cast<int>(sizeof(double2));
     return cudaFuncSetAttribute(k_diaginv<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm64);
@@ -565,7 +711,7 @@ cudaError_t launch_accumulate(const Plan& P, const DevTables& T, const Workspace
         count = P.nnz;
     }
     const int blocks = accumulate_blocks(count);
-    k_accumulate<<<blocks, kAccThreads, 0, st>>>(T.out_map, k0, count, W.fronts, W.front_stride, np, c, S, rho,
+    k_accumulate<<<blocks, kAccThreads, 0, st>>>(T.out_map, W.scale_pair, k0, count, W.fronts, W.front_stride, np, c, S, rho,
                                                  accumulate, want_trace, partials);
     return cudaGetLastError();
 }
@@ -608,14 +754,15 @@ double gershgorin_value(unsigned long long key) {
     return x;
 }
 
-__global__ void __launch_bounds__(kAccThreads) k_point_traces(const int64_t* __restrict__ out_map, int64_t nnz,
+__global__ void __launch_bounds__(kAccThreads) k_point_traces(const int64_t* __restrict__ out_map,
+                                                              const int16_t* __restrict__ pair, int64_t nnz,
                                                               const double2* __restrict__ F, int64_t stride,
                                                               const double* __restrict__ S,
                                                               double* __restrict__ partials) {
     __shared__ double red[kAccThreads / 32];
     const int64_t k = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
     double v = 0.0;
-    if (k < nnz) v = F[static_cast<int64_t>(blockIdx.y) * stride + out_map[k]].y * S[k];
+    if (k < nnz) v = scale2(F[static_cast<int64_t>(blockIdx.y) * stride + out_map[k]].y, pair[k]) * S[k];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
@@ -628,12 +775,13 @@ __global__ void __launch_bounds__(kAccThreads) k_point_traces(const int64_t* __r
     }
 }
 
-cudaError_t launch_point_traces_range(const int64_t* out_map, int64_t nnz, const double2* F, int64_t stride, int np,
-                                      const double* S, double* partials, double* out, cudaStream_t st) {
+cudaError_t launch_point_traces_range(const int64_t* out_map, const int16_t* pair, int64_t nnz, const double2* F,
+                                      int64_t stride, int np, const double* S, double* partials, double* out,
+                                      cudaStream_t st) {
     if (nnz <= 0 || np <= 0) return cudaSuccess;
     const int nb = accumulate_blocks(nnz);
     k_point_traces<<<dim3(static_cast<unsigned>(nb), static_cast<unsigned>(np)), kAccThreads, 0, st>>>(
-        out_map, nnz, F, stride, S, partials);
+        out_map, pair, nnz, F, stride, S, partials);
     cudaError_t e = cudaGetLastError();
     for (int q = 0; q < np && e == cudaSuccess; ++q) {
         k_reduce<<<1, 1024, 0, st>>>(partials + static_cast<int64_t>(q) * nb, nb, out + q);
@@ -644,7 +792,7 @@ cudaError_t launch_point_traces_range(const int64_t* out_map, int64_t nnz, const
 
 cudaError_t launch_point_traces(const Plan& P, const DevTables& T, const Workspace& W, int np, const double* S,
                                 double* partials, double* out, cudaStream_t st) {
-    return launch_point_traces_range(T.out_map, P.nnz, W.fronts, W.front_stride, np, S, partials, out, st);
+    return launch_point_traces_range(T.out_map, W.scale_pair, P.nnz, W.fronts, W.front_stride, np, S, partials, out, st);
 }
 
 cudaError_t launch_reduce(const double* partials, int nblocks, double* out, cudaStream_t st) {
@@ -656,7 +804,7 @@ cudaError_t launch_gather_pattern(const Plan& P, const DevTables& T, const Works
                                   double2* G_out, int64_t q0, cudaStream_t st) {
     const int64_t blocks = (P.nnz + 255) / 256;
     dim3 grid(static_cast<unsigned>(blocks < 2048 ? blocks : 2048), static_cast<unsigned>(np));
-    k_gather_pattern<<<grid, 256, 0, st>>>(T.out_map, P.nnz, W.fronts, W.front_stride, G_out, q0);
+    k_gather_pattern<<<grid, 256, 0, st>>>(T.out_map, W.scale_pair, P.nnz, W.fronts, W.front_stride, G_out, q0);
     return cudaGetLastError();
 }
 

@@ -38,7 +38,21 @@ struct Workspace {
     int64_t front_stride = 0;   // complex elements per pole slab
     int64_t scr_stride = 0;
     int32_t np_cap = 0;         // poles the buffers hold
+    // Power-of-two scaling of the basis functions the fronts were assembled with (part of the fronts'
+    // allocation): exponent f_i per basis function, f_i + f_j per pattern entry, any f_i != 0.
+    int16_t* scale_f = nullptr;
+    int16_t* scale_pair = nullptr;
+    int* scale_any = nullptr;
 };
+
+// Bytes of the scaling tables behind the fronts.
+inline size_t scale_bytes(const Plan& P) { return 256 + sizeof(int16_t) * static_cast<size_t>(P.n + P.nnz); }
+
+// Fill the scaling tables of W from the diagonal of S (values on the pattern): 2^f_i brings S_ii into
+// [1/2, 2).  The fronts hold D (z S - H) D with D = diag(2^f_i), exactly, and so D^{-1} G D^{-1}: a
+// basis whose functions are normalised very differently does not leave rows of mixed scale for the
+// fixed-point and split products.  Outputs take the pair exponents (solves the row exponents) again.
+cudaError_t launch_basis_scale(const Plan& P, const DevTables& T, const double* S, const Workspace& W, cudaStream_t st);
 
 // Spectral-moment features of (H, S) for the learned mu seed (mlp.cu).
 int mlp_features(const Plan& P, const double* Hd, const double* Sd, const int64_t* rowptr_d,
@@ -73,9 +87,10 @@ double gershgorin_value(unsigned long long key);
 // Per point q of a chunk: out[q] = sum over the pattern of Im G_q(k) S_k = Im Tr(G(z_q) S) (the
 // density of states of Eq. 42 up to -2/pi).  partials: np x accumulate_blocks(nnz) doubles.
 // The same over one range of pattern entries (out_map and S offset to its first entry; F holds np
-// point slabs of `stride` complex elements): out[q] = sum_k Im F_q[out_map[k]] S[k].
-cudaError_t launch_point_traces_range(const int64_t* out_map, int64_t nnz, const double2* F, int64_t stride, int np,
-                                      const double* S, double* partials, double* out, cudaStream_t st);
+// point slabs of `stride` complex elements): out[q] = sum_k Im F_q[out_map[k]] 2^pair[k] S[k].
+cudaError_t launch_point_traces_range(const int64_t* out_map, const int16_t* pair, int64_t nnz, const double2* F,
+                                      int64_t stride, int np, const double* S, double* partials, double* out,
+                                      cudaStream_t st);
 cudaError_t launch_point_traces(const Plan& P, const DevTables& T, const Workspace& W, int np,
                                 const double* S, double* partials, double* out, cudaStream_t st);
 

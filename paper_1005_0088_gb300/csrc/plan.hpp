@@ -75,7 +75,7 @@ struct Launch {
     double alpha, beta;
     int64_t first, count;    // range in the item array of this kind
     int64_t tfirst, tcount;  // GEMM tiles range
-    int32_t tile;            // FP64 GEMM output tile edge (16 or 32); pivot-sweep width of a diag launch
+    int32_t tile;            // FP64 GEMM output tile edge; pivot-sweep width of a diag launch
     int32_t exact;           // 1: FP64 CUDA-core GEMM in every precision mode (diagonal blocks)
     int32_t phase;           // 0 factor, 1 selinv
     int32_t tag;             // which formula the step implements (for profiling names)
@@ -175,8 +175,7 @@ int mu_search_batched(int32_t ns, ndsi_mu_eval_batch_fn eval, ndsi_mu_dos_batch_
 int cf_poles(int32_t M, double* z, double* R, std::string& err);
 
 // Tile sizes shared by the schedule and the kernels.
-constexpr int kGemmTile = 32;     // largest FP64 GEMM output tile (rows and columns)
-constexpr int kGemmTileSmall = 16;  // output tile for launches whose items are small
+constexpr int kGemmTile = 32;     // FP64 GEMM output tile (rows and columns)
 constexpr int kNodeTile = 32;     // assembly / gather tile
 
 void set_last_error(const std::string& msg);

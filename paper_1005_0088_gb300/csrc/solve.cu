@@ -180,6 +180,15 @@ __global__ void __launch_bounds__(kSolveThreads) k_solve_bwd(const SolveNode* __
         if (kRq * q + u < nc) atomic_add2(dst + kRq * q + u, acc.get(u, -1.0));
 }
 
+// Row i of the n x k block X times 2^f_i.
+__global__ void __launch_bounds__(256) k_scale_rows(const int16_t* __restrict__ f, int64_t count, int k,
+                                                    double2* __restrict__ X) {
+    const int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (e >= count) return;
+    const int s = f[e / k];
+    if (s != 0) X[e] = make_double2(ldexp(X[e].x, s), ldexp(X[e].y, s));
+}
+
 // One warp per row of the CSR matrix, lanes over the m columns.
 __global__ void __launch_bounds__(256) k_spmm(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
                                               const double* __restrict__ A, int64_t n,
@@ -422,7 +431,7 @@ constexpr size_t kFwdSmem = sizeof(double2) * kT * kTP + 2 * sizeof(RhsTile);
 constexpr size_t kBwdSmem = sizeof(double2) * kT * kTP + sizeof(RhsTile);
 
 cudaError_t launch_solve(const Plan& P, const SolveTables& T, const double2* fronts, double2* Y, double2* X, int k,
-                         cudaStream_t st) {
+                         const int16_t* scale_f, cudaStream_t st) {
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(k_solve_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   static_cast<int>(kFwdSmem))) != cudaSuccess)
@@ -433,6 +442,12 @@ cudaError_t launch_solve(const Plan& P, const SolveTables& T, const double2* fro
     const unsigned gy = static_cast<unsigned>((k + kSolveRhs - 1) / kSolveRhs);
     e = cudaMemsetAsync(X, 0, sizeof(double2) * static_cast<size_t>(P.n) * k, st);
     if (e != cudaSuccess) return e;
+    const int64_t count = P.n * static_cast<int64_t>(k);
+    auto scale_rows = [&](double2* B) {
+        if (scale_f) k_scale_rows<<<static_cast<unsigned>((count + 255) / 256), 256, 0, st>>>(scale_f, count, k, B);
+        return cudaGetLastError();
+    };
+    if ((e = scale_rows(Y)) != cudaSuccess) return e;
     for (int32_t L = 0; L < P.n_levels; ++L) {
         const int64_t cnt = T.fwd_first[L + 1] - T.fwd_first[L];
         if (cnt == 0) continue;
@@ -447,7 +462,7 @@ cudaError_t launch_solve(const Plan& P, const SolveTables& T, const double2* fro
                                                                            X, k);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    return cudaSuccess;
+    return scale_rows(X);
 }
 
 cudaError_t launch_spmm(const int64_t* rowptr, const int32_t* col, const double* A, int64_t n, const double* X,

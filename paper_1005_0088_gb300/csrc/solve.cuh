@@ -47,8 +47,10 @@ void solve_tables_free(SolveTables& T);
 // n x k, row-major (the k right-hand sides of a basis index are adjacent), original basis order.
 // Y is overwritten (the forward elimination works in it).  Every tile accumulates into X and Y
 // with FP64 atomics, so the rounding order (not the result beyond it) varies from run to run.
+// scale_f: exponents of the basis scaling of the factors (the rows of Y and of X are multiplied by
+// 2^f), or NULL when all are 0.
 cudaError_t launch_solve(const Plan& P, const SolveTables& T, const double2* fronts, double2* Y, double2* X, int k,
-                         cudaStream_t st);
+                         const int16_t* scale_f, cudaStream_t st);
 
 // Y[:, 0:m] = A X[:, 0:m] for the real CSR matrix A on the pattern (values in pattern order);
 // X and Y are n x ld row-major.

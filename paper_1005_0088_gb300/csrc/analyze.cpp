@@ -646,8 +646,57 @@ void build_schedule(Plan& P) {
         int32_t nob = 0;
         for (int32_t j : nodesL) nob = std::max<int32_t>(nob, static_cast<int32_t>(ceil_div(P.s[j], Bo)));
         for (int32_t T = 0; T < nob; ++T) {
+            // (i+ii) in one launch: the whole block inverted in shared memory (k_diaginv_block), for
+            // the default pivot width and blocks that fit; widest blocks first, so that the last
+            // ones to start are the short ones
+            const bool fused = b == 16 && Bo <= kDiagBlockMax;
+            if (fused) {
+                std::vector<DiagItem> its;
+                for (int32_t j : nodesL) {
+                    const int32_t s = P.s[j], f = P.f[j];
+                    const int32_t K0 = T * Bo;
+                    if (K0 >= s) continue;
+                    its.push_back(DiagItem{P.front_off[j] + K0 + static_cast<int64_t>(K0) * f, f, std::min(Bo, s - K0)});
+                }
+                std::stable_sort(its.begin(), its.end(),
+                                 [](const DiagItem& x, const DiagItem& y) { return x.nb > y.nb; });
+                // One launch per width class (the classes of k_diaginv_block's occupancy), so that narrow
+                // blocks do not take the shared memory of wide ones; a class of few blocks stays with
+                // the wider ones, where it costs no launch of its own.
+                size_t i0 = 0;
+                while (i0 < its.size()) {
+                    size_t i1 = its.size();
+                    for (const int32_t w : {80, 64}) {
+                        size_t c = i0;
+                        while (c < its.size() && its[c].nb > w) ++c;
+                        if (c > i0 && its.size() - c >= kDiagClassMin) {
+                            i1 = c;
+                            break;
+                        }
+                    }
+                    Launch ld = new_launch(L_DIAGINV, L, 0, T_DINV);
+                    ld.first = static_cast<int64_t>(P.diag_items.size());
+                    ld.count = static_cast<int64_t>(i1 - i0);
+                    ld.tile = (its[i0].nb + 15) / 16 * 16;
+                    ld.fused = ld.tile > 16 ? 1 : 0;  // single pivot blocks: one warp each
+                    for (size_t i = i0; i < i1; ++i) {
+                        const int32_t n = its[i].nb;
+                        P.diag_items.push_back(its[i]);
+                        ld.bytes += 16.0 * n * (n + 1.0);
+                        // algorithmic flops of the block LDL^T and the inverse by 16-wide pivot blocks
+                        for (int32_t k0 = 0; k0 < n; k0 += b) {
+                            const double w = std::min(b, n - k0), m = n - k0 - w;
+                            ld.flops += 8.0 * (w * w * w + m * w * w + 0.5 * m * (m + 1.0) * w + m * m * w +
+                                               0.5 * w * (w + 1.0) * m);
+                        }
+                    }
+                    P.flops_per_pole += ld.flops;
+                    P.launches.push_back(ld);
+                    i0 = i1;
+                }
+            }
             // (i) block LDL^T of diagonal block T in pivot blocks of b
-            for (int32_t t = 0; t < Bo / b; ++t) {
+            for (int32_t t = 0; !fused && t < Bo / b; ++t) {
                 Launch ld = new_launch(L_DIAGINV, L, 0, T_DINV);
                 ld.first = static_cast<int64_t>(P.diag_items.size());
                 std::vector<GSpec> panel, update;
@@ -688,7 +737,7 @@ void build_schedule(Plan& P) {
                 emit_copy(L, 0, T_PCOPY, 1.0, copies);
             }
             // (ii) inverse of diagonal block T in place, from its pivot blocks backwards
-            for (int32_t t = Bo / b - 1; t >= 0; --t) {
+            for (int32_t t = fused ? -1 : Bo / b - 1; t >= 0; --t) {
                 std::vector<GSpec> tg, dg;
                 std::vector<CopyItem> copies;
                 for (int32_t j : nodesL) {

@@ -218,7 +218,7 @@ int run_phase(ndsi_plan* h, const Workspace& W, const SplitBuffers& SB, int phas
                     h->SP.tensor_flops[si] * np * pair_frac);
         } else {
             e = timed(h->prof,
-                      family_of(l) + (h->prof.by_level && l.kind == L_GEMM ? ":L" + std::to_string(l.level) : std::string()),
+                      family_of(l) + (h->prof.by_level && (l.kind == L_GEMM || l.kind == L_DIAGINV) ? ":L" + std::to_string(l.level) : std::string()),
                       l.flops * np, l.bytes * np, st,
                       [&]() { return launch_step(P, h->T, l, W, H, S, z, zstride, np, st); });
         }

@@ -250,19 +250,20 @@ __global__ void __launch_bounds__(32) k_diaginv_sweep(const DiagItem* __restrict
         __syncwarp();
         const double2 p = cs[t];
         const double den = p.x * p.x + p.y * p.y;
-        bad |= !(den > 0.0 && isfinite(den));
+        bad |= (static_cast<uint32_t>(__double2hiint(den)) >> 20) - 1u >= 0x7FEu;  // zero, subnormal, non-finite
         const double rden = 1.0 / den;
-        const double2 ip = make_double2(p.x * rden, -p.y * rden);
+        const double2 ip = make_double2(p.x * rden, -p.y * rden), nip = make_double2(-ip.x, -ip.y);
         if (lane < N) ds[lane] = cmul(cs[lane], ip);
         __syncwarp();
 #pragma unroll
         for (int s = 0; s < SLOTS; ++s) {
             const int i = rc[s] & 255, k = rc[s] >> 8;
-            const double2 cv = cs[i], dk = ds[k];
-            double2 g = make_double2(a[s].x - (cv.x * dk.x - cv.y * dk.y), a[s].y - (cv.x * dk.y + cv.y * dk.x));
-            if (k == t) g = i == t ? make_double2(-ip.x, -ip.y) : ds[i];
-            else if (i == t) g = dk;
-            a[s] = g;
+            const double2 cv = cs[i], dk = ds[k], di = ds[i];
+            const double2 g = make_double2(fma(-cv.x, dk.x, fma(cv.y, dk.y, a[s].x)), fma(-cv.x, dk.y, fma(-cv.y, dk.x, a[s].y)));
+            // the pivot row and column take d (the pivot itself -1/p), by selects: a branch here diverges
+            const bool kq = k == t, iq = i == t;
+            const double2 o = kq ? (iq ? nip : di) : dk;
+            a[s] = make_double2(kq | iq ? o.x : g.x, kq | iq ? o.y : g.y);
         }
         __syncwarp();
     }
@@ -359,6 +360,306 @@ __device__ __forceinline__ int4 fix_digits2(double2 v, int emax) {
 }
 // Exponent a row's digits are stored with, from its largest exponent field.
 __device__ __forceinline__ int fix_expo(int emax) { return emax == 0x7FF ? kFixNonFinite : emax - 1022 - 57; }
+
+// ---------------------------------------------------------------------------------------------
+// Whole diagonal block in one launch: the inverse of a complex-symmetric block of up to 128 columns
+// by the symmetric block sweep.  With pivot block t (16 wide), P = A_tt^{-1}, C_i = A_it and
+// W_i = C_i P the sweep maps
+//     A_ij <- A_ij - W_i C_j^T (i, j outside the pivot),   A_it <- W_i,   A_tt <- -P,
+// and after every pivot block A holds -A^{-1}; every intermediate matrix is symmetric, so only 8 x 8
+// blocks of the lower triangle are kept (in shared memory, FP64) and updated (n^3 / 2 complex
+// multiply-adds).  The pivot blocks are inverted in FP64; the panel and update products run in
+// fixed point (above), with the panels' digits formed once per pivot step.
+// Bound: the integer multiply-add pipe for the updates (16 x 8 units handed out dynamically) and the
+// FP64 latency of the pivot block (16 dependent divisions, about 40k clocks on one warp, since a
+// sub-partition takes 64 clocks per FP64 instruction); one warp therefore inverts the next pivot
+// block, updated first, while the others still update.
+// Replaces, per 16 columns, a pivot-inverse, panel, update and copy launch each and the backward
+// assembly (53 launches for 128 columns).
+constexpr int kBlkP = 16;  // pivot width
+
+__host__ __device__ constexpr size_t diag_block_smem(int tile) {
+    const int nb8 = tile / 8, rows = tile - kBlkP;
+    return static_cast<size_t>(nb8 * (nb8 + 1) / 2) * 64 * sizeof(double2) +        // lower 8 x 8 blocks
+           sizeof(int4) * (2 * kBlkP * rows + kBlkP * kBlkP) +                      // digits of W, C and P
+           sizeof(int) * (2 * rows + kBlkP) + sizeof(double2) * 2 * (kBlkP + 1) +   // exponents, pivot column
+           sizeof(int) * 4 + sizeof(uint16_t) * nb8 * (nb8 + 1) / 2;                // counters, unit list
+}
+
+// Threads per block of up to `tile` columns: narrow blocks leave room for three CTAs (64 columns, 65 KB
+// each) or two (80 columns) on an SM, whose pivot inversions then overlap; a 128-column block fills
+// one SM's shared memory and uses 16 warps for its updates.
+constexpr int diag_block_threads(int tile) { return tile <= 64 ? 128 : tile <= 80 ? 256 : 512; }
+
+__global__ void __launch_bounds__(512) k_diaginv_block(const DiagItem* __restrict__ items, int64_t first,
+                                                       double2* __restrict__ F, int64_t stride,
+                                                       int* __restrict__ status, int tile) {
+    extern __shared__ double2 smem_blk[];
+    const int T8 = tile / 8, R = tile - kBlkP;
+    double2* M = smem_blk;                                    // block (I, J) at I (I + 1) / 2 + J, column-major
+    int4* Wd = reinterpret_cast<int4*>(M + (T8 * (T8 + 1) / 2) * 64);  // [16][R], k-major
+    int4 *Cd = Wd + kBlkP * R, *Pd = Cd + kBlkP * R;          // [16][R]; [16][16] symmetric
+    double2* cs = reinterpret_cast<double2*>(Pd + kBlkP * kBlkP);      // [17] pivot column, [16] dummy
+    double2* ds = cs + kBlkP + 1;
+    int* We = reinterpret_cast<int*>(ds + kBlkP + 1);         // row exponents of W, C; column exponents of P
+    int *Ce = We + R, *Pe = Ce + R;
+    int* ctr = Pe + kBlkP;                                    // [0] next unit, [1] list length
+    uint16_t* list = reinterpret_cast<uint16_t*>(ctr + 4);    // update units: row pair I16 << 8 | column block J
+    const DiagItem d = items[first + blockIdx.x];
+    double2* A = F + static_cast<int64_t>(blockIdx.y) * stride + d.off;
+    const int n = d.nb, ld = d.ld;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    if (n > tile) {
+        if (tid == 0) atomicOr(status, kStatusBadItem);
+        return;
+    }
+    const int nb8 = (n + 7) / 8, nt = (n + kBlkP - 1) / kBlkP;
+    auto blk = [&](int I, int J) { return M + (I * (I + 1) / 2 + J) * 64; };
+    // load the lower triangle (rows and columns past n are zero)
+    for (int b = warp; b < nb8 * (nb8 + 1) / 2; b += nw) {
+        int I = 0;
+        while ((I + 1) * (I + 2) / 2 <= b) ++I;
+        const int J = b - I * (I + 1) / 2;
+        for (int e = lane; e < 64; e += 32) {
+            const int i = I * 8 + (e & 7), j = J * 8 + (e >> 3);
+            M[b * 64 + e] = (i < n && j <= i) ? A[i + static_cast<int64_t>(j) * ld] : make_double2(0.0, 0.0);
+        }
+    }
+    if (tid == 0) {
+        int cnt = 0;
+        for (int I = 0; I < nt; ++I)
+            for (int J = 0; J <= min(2 * I + 1, nb8 - 1); ++J) list[cnt++] = static_cast<uint16_t>(I << 8 | J);
+        ctr[1] = cnt;
+    }
+    const int r8 = lane & 7, cq = lane >> 3;  // a unit's row and first column of this lane
+    // inverse of pivot block t by one warp (rank-1 symmetric sweeps, packed lower triangle; see
+    // k_diaginv_sweep), written to the block itself (-P) and, as digits, to P
+    auto pivot = [&](int t) {
+        constexpr int VC = kBlkP / 2, LPC = 32 / VC, SLOTS = (kBlkP + 1 + LPC - 1) / LPC;
+        const int nb = min(kBlkP, n - t * kBlkP);
+        const int c = lane % VC, vbase = (lane / VC) * SLOTS;
+        auto at = [&](int i, int k) { return blk(2 * t + (i >> 3), 2 * t + (k >> 3)) + (k & 7) * 8 + (i & 7); };
+        int rc[SLOTS];
+        double2 a[SLOTS];
+#pragma unroll
+        for (int s = 0; s < SLOTS; ++s) {
+            const int v = vbase + s;
+            int i = kBlkP, k = kBlkP;
+            if (v < kBlkP - c) {
+                i = c + v;
+                k = c;
+            } else if (v <= kBlkP) {
+                i = v - 1;
+                k = kBlkP - 1 - c;
+            }
+            rc[s] = i | (k << 8);
+            a[s] = make_double2(0.0, 0.0);
+            if (i < nb && k < nb) a[s] = *at(i, k);
+        }
+        if (lane == 0) cs[kBlkP] = ds[kBlkP] = make_double2(0.0, 0.0);
+        bool bad = false;
+        for (int q = 0; q < nb; ++q) {
+#pragma unroll
+            for (int s = 0; s < SLOTS; ++s) {
+                const int i = rc[s] & 255, k = rc[s] >> 8;
+                if (k == q) cs[i] = a[s];
+                if (i == q) cs[k] = a[s];
+            }
+            __syncwarp();
+            const double2 p = cs[q];
+            const double den = p.x * p.x + p.y * p.y;
+            // zero, subnormal or non-finite: decided on the exponent field, off the FP64 pipe
+            const uint32_t dx = static_cast<uint32_t>(__double2hiint(den)) >> 20;
+            bad |= dx - 1u >= 0x7FEu;
+            const double rden = 1.0 / den;
+            const double2 ip = make_double2(p.x * rden, -p.y * rden), nip = make_double2(-ip.x, -ip.y);
+            if (lane < kBlkP) ds[lane] = cmul(cs[lane], ip);
+            __syncwarp();
+#pragma unroll
+            for (int s = 0; s < SLOTS; ++s) {
+                const int i = rc[s] & 255, k = rc[s] >> 8;
+                const double2 cv = cs[i], dk = ds[k], di = ds[i];
+                const double2 g = make_double2(fma(-cv.x, dk.x, fma(cv.y, dk.y, a[s].x)), fma(-cv.x, dk.y, fma(-cv.y, dk.x, a[s].y)));
+                // the pivot row and column take d (the pivot itself -1/p), by selects: a branch here diverges
+                const bool kq = k == q, iq = i == q;
+                const double2 o = kq ? (iq ? nip : di) : dk;
+                a[s] = make_double2(kq | iq ? o.x : g.x, kq | iq ? o.y : g.y);
+            }
+            __syncwarp();
+        }
+        if (bad && lane == 0) atomicOr(status, kStatusSingular);
+        double2* P = reinterpret_cast<double2*>(Pd);
+#pragma unroll
+        for (int s = 0; s < SLOTS; ++s) {
+            const int i = rc[s] & 255, k = rc[s] >> 8;
+            if (i >= kBlkP) continue;
+            const bool in = i < nb && k < nb;
+            if (in) *at(i, k) = a[s];
+            P[i * kBlkP + k] = P[k * kBlkP + i] = in ? make_double2(-a[s].x, -a[s].y) : make_double2(0.0, 0.0);
+        }
+        __syncwarp();
+        // digits of P in place, two lanes per column
+        const int col = lane & 15, kh = lane >> 4;
+        int emax = 0;
+#pragma unroll
+        for (int k = 0; k < kBlkP / 2; ++k) emax = max(emax, expo_bits(P[(2 * k + kh) * kBlkP + col]));
+        emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 16)) >> 20;
+#pragma unroll
+        for (int k = 0; k < kBlkP / 2; ++k) {
+            const int o = (2 * k + kh) * kBlkP + col;
+            Pd[o] = fix_digits2(P[o], emax);
+        }
+        if (kh == 0) Pe[col] = fix_expo(emax);
+    };
+    __syncthreads();
+    // the warp that inverts the pivot blocks: co-resident CTAs take warps of different SM sub-partitions
+    uint32_t slot;
+    asm volatile("mov.u32 %0, %%warpid;" : "=r"(slot));
+    if (tid == 0) ctr[2] = static_cast<int>(slot / nw) & 3;
+    __syncthreads();
+    const int wp = ctr[2];
+    if (warp == wp) pivot(0);
+    __syncthreads();
+    for (int t = 0; t < nt; ++t) {
+        const int w8 = min(2, nb8 - 2 * t), kw = 8 * w8, m8 = nb8 - w8, m = 8 * m8;
+        // digits of the pivot column: panel row `row` is matrix row row (above the pivot) or
+        // row + kw; two threads per row
+        if (tid == 0) ctr[0] = 0;
+        for (int r0 = warp * 16; r0 < m; r0 += nw * 16) {
+            const int row = r0 + (lane & 15), kh = lane >> 4;
+            const int I = row >> 3, Ig = I < 2 * t ? I : I + w8, r = row & 7;
+            double2 v[kBlkP / 2];
+            int emax = 0;
+#pragma unroll
+            for (int k = 0; k < kBlkP / 2; ++k) {
+                v[k] = make_double2(0.0, 0.0);
+                if (row < m && 2 * k < kw) {
+                    const int kk = 2 * k + kh, K = 2 * t + (kk >> 3);
+                    v[k] = Ig < K ? blk(K, Ig)[r * 8 + (kk & 7)] : blk(Ig, K)[(kk & 7) * 8 + r];
+                }
+                emax = max(emax, expo_bits(v[k]));
+            }
+            emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 16)) >> 20;
+            if (row < m) {
+#pragma unroll
+                for (int k = 0; k < kBlkP / 2; ++k)
+                    if (2 * k < kw) Cd[(2 * k + kh) * R + row] = fix_digits2(v[k], emax);
+                if (kh == 0) Ce[row] = fix_expo(emax);
+            }
+        }
+        __syncthreads();
+        // W = C P, eight rows of W per warp; the pivot column becomes W (its old values stay in C)
+        for (int u = warp; u < m8; u += nw) {
+            const int row = u * 8 + r8, Ig = u < 2 * t ? u : u + w8;
+            FixSum c[4] = {};
+#pragma unroll 2
+            for (int k = 0; k < kw; ++k) {
+                const int4 a = Cd[k * R + row];
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (4 * q < kw) fix_mac(c[q], a, Pd[k * kBlkP + cq + 4 * q]);
+            }
+            double2 w[4];
+            int emax = 0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                w[q] = make_double2(0.0, 0.0);
+                if (4 * q < kw) w[q] = fix_value(c[q], Ce[row] + Pe[cq + 4 * q]);
+                emax = max(emax, expo_bits(w[q]));
+            }
+            emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 8));
+            emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 16)) >> 20;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (4 * q >= kw) continue;
+                const int k = cq + 4 * q, K = 2 * t + (k >> 3);
+                Wd[k * R + row] = fix_digits2(w[q], emax);
+                (Ig < K ? blk(K, Ig)[r8 * 8 + (k & 7)] : blk(Ig, K)[(k & 7) * 8 + r8]) = w[q];
+            }
+            if (cq == 0) We[row] = fix_expo(emax);
+        }
+        __syncthreads();
+        // A_IJ -= W_I C_J^T for the row blocks 2 I16, 2 I16 + 1 and column block J, one unit per warp
+        auto update = [&](int I16, int J) {
+            const int I0 = 2 * I16, shift = I0 < 2 * t ? 0 : w8;
+            const bool lo = J <= I0, hi = I0 + 1 < nb8;
+            const int row = (I0 - shift) * 8 + r8, col = (J < 2 * t ? J : J - w8) * 8 + cq;
+            FixSum c[2][2] = {};
+            if (lo && hi) {
+#pragma unroll 2
+                for (int k = 0; k < kw; ++k) {
+                    const int4 a0 = Wd[k * R + row], a1 = Wd[k * R + row + 8];
+                    const int4 b0 = Cd[k * R + col], b1 = Cd[k * R + col + 4];
+                    fix_mac(c[0][0], a0, b0);
+                    fix_mac(c[0][1], a0, b1);
+                    fix_mac(c[1][0], a1, b0);
+                    fix_mac(c[1][1], a1, b1);
+                }
+            } else {
+                const int r = lo ? row : row + 8, g = lo ? 0 : 1;
+                FixSum c0{}, c1{};
+#pragma unroll 2
+                for (int k = 0; k < kw; ++k) {
+                    const int4 a = Wd[k * R + r];
+                    fix_mac(c0, a, Cd[k * R + col]);
+                    fix_mac(c1, a, Cd[k * R + col + 4]);
+                }
+                if (g == 0) c[0][0] = c0, c[0][1] = c1;
+                else c[1][0] = c0, c[1][1] = c1;
+            }
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                if (g == 0 ? !lo : !hi) continue;
+                double2* dst = blk(I0 + g, J);
+                const int ea = We[row + 8 * g];
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const double2 p = fix_value(c[g][q], ea + Ce[col + 4 * q]);
+                    double2& v = dst[(cq + 4 * q) * 8 + r8];
+                    v = make_double2(v.x - p.x, v.y - p.y);
+                }
+            }
+        };
+        // the next pivot block is updated first, in six 8 x 4 pieces over the warps, and one warp
+        // inverts it while the others update the rest
+        const bool ahead = t + 1 < nt;
+        if (ahead) {
+            const int N0 = 2 * t + 2;
+            for (int u = warp; u < 6; u += nw) {
+                const int I = N0 + (u >= 2), J = N0 + (u >= 4);  // (0,0) (1,0) (1,1) of the pivot block
+                if (I >= nb8) continue;
+                const int row = (I - w8) * 8 + r8, c4 = cq + 4 * (u & 1), col = (J - w8) * 8 + c4;
+                FixSum c{};
+#pragma unroll 2
+                for (int k = 0; k < kw; ++k) fix_mac(c, Wd[k * R + row], Cd[k * R + col]);
+                const double2 p = fix_value(c, We[row] + Ce[col]);
+                double2& v = blk(I, J)[c4 * 8 + r8];
+                v = make_double2(v.x - p.x, v.y - p.y);
+            }
+            __syncthreads();
+            if (warp == wp) pivot(t + 1);
+        }
+        const int cnt = ctr[1];
+        while (true) {
+            int u = lane == 0 ? atomicAdd(&ctr[0], 1) : 0;
+            u = __shfl_sync(0xffffffffu, u, 0);
+            if (u >= cnt) break;
+            const int I = list[u] >> 8, J = list[u] & 255;
+            if (I == t || (J >> 1) == t || (ahead && I == t + 1 && (J >> 1) == t + 1)) continue;
+            update(I, J);
+        }
+        __syncthreads();
+    }
+    for (int b = warp; b < nb8 * (nb8 + 1) / 2; b += nw) {
+        int I = 0;
+        while ((I + 1) * (I + 2) / 2 <= b) ++I;
+        const int J = b - I * (I + 1) / 2;
+        for (int e = lane; e < 64; e += 32) {
+            const int i = I * 8 + (e & 7), j = J * 8 + (e >> 3);
+            if (i < n && j <= i) A[i + static_cast<int64_t>(j) * ld] = make_double2(-M[b * 64 + e].x, -M[b * 64 + e].y);
+        }
+    }
+}
 
 // ---------------------------------------------------------------------------------------------
 // Batched complex FP64 GEMM on the CUDA cores: C = alpha op(A) op(B) + beta C for every tile of
@@ -648,6 +949,12 @@ cudaError_t launch_step(const Plan& P, const DevTables& T, const Launch& l, cons
             return cudaGetLastError();
         }
         case L_DIAGINV: {
+            if (l.fused) {
+                k_diaginv_block<<<dim3(static_cast<unsigned>(l.count), static_cast<unsigned>(np)), diag_block_threads(l.tile),
+                                  diag_block_smem(l.tile), st>>>(T.diag_items, l.first, W.fronts, W.front_stride, T.status,
+                                                                 l.tile);
+                return cudaGetLastError();
+            }
             dim3 grid(static_cast<unsigned>(l.count), static_cast<unsigned>(np));
             const int b = P.block;
             const size_t sm = static_cast<size_t>(b) * (b + 1) * sizeof(double2);
@@ -697,6 +1004,9 @@ cudaError_t launch_basis_scale(const Plan& P, const DevTables& T, const double* 
 }
 
 cudaError_t kernels_init() {
+    const int smb = static_cast<int>(diag_block_smem(kDiagBlockMax));
+    const cudaError_t e = cudaFuncSetAttribute(k_diaginv_block, cudaFuncAttributeMaxDynamicSharedMemorySize, smb);
+    if (e != cudaSuccess) return e;
     const int sm64 = 64 * 65 * static_cast<int>(sizeof(double2));
     return cudaFuncSetAttribute(k_diaginv<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm64);
 }

@@ -75,8 +75,9 @@ struct Launch {
     double alpha, beta;
     int64_t first, count;    // range in the item array of this kind
     int64_t tfirst, tcount;  // GEMM tiles range
-    int32_t tile;            // FP64 GEMM output tile edge; pivot-sweep width of a diag launch
+    int32_t tile;            // FP64 GEMM output tile edge; widest block a diag launch inverts
     int32_t exact;           // 1: FP64 CUDA-core GEMM in every precision mode (diagonal blocks)
+    int32_t fused;           // diag launch: 1 = whole diagonal blocks of up to `tile` columns each
     int32_t phase;           // 0 factor, 1 selinv
     int32_t tag;             // which formula the step implements (for profiling names)
     double flops;            // algorithmic real flops per pole of this launch
@@ -177,6 +178,8 @@ int cf_poles(int32_t M, double* z, double* R, std::string& err);
 // Tile sizes shared by the schedule and the kernels.
 constexpr int kGemmTile = 32;     // FP64 GEMM output tile (rows and columns)
 constexpr int kNodeTile = 32;     // assembly / gather tile
+constexpr size_t kDiagClassMin = 16;  // blocks of a width class that get a launch of their own
+constexpr int kDiagBlockMax = 128;  // widest diagonal block the one-launch inverse holds in shared memory
 
 void set_last_error(const std::string& msg);
 

@@ -198,9 +198,11 @@ struct Checker {
                 Writes W;
                 if (!build_writes(writes, W, tag)) return false;
             } else if (l.kind == L_DIAGINV) {
-                // widest block the launch's kernel inverts: warp sweeps of 16 or 32, else the
-                // shared-memory kernel of 64
-                const int32_t cap = P.block <= 32 ? (l.tile == 16 ? 16 : 32) : 64;
+                // widest block the launch's kernel inverts: a whole diagonal block of up to `tile`
+                // columns, warp sweeps of 16 or 32, else the shared-memory kernel of 64
+                const int32_t cap = l.fused ? l.tile : P.block <= 32 ? (l.tile == 16 ? 16 : 32) : 64;
+                if (l.fused && (l.tile <= 16 || l.tile > kDiagBlockMax || l.tile % 16))
+                    return fail("diagonal-block launch of an unsupported width (" + tag + ")");
                 for (int64_t i = l.first; i < l.first + l.count; ++i) {
                     const DiagItem& d = P.diag_items[i];
                     Region D;

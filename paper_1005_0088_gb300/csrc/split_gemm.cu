@@ -15,21 +15,37 @@
 //    consecutive rows of one K-major block, so A_t times [B_1; ...; B_{S+1-t}] is one wide MMA (or
 //    two, N <= 256) whose output columns fall into the accumulators of t+1 .. S+1 - each operand
 //    tile is read from shared memory once per digit instead of once per product, which keeps
-//    the tensor pipe fed at N = 2NC = 80.  Within an accumulator every partial sum over a
-//    256-element K chunk has at most four products per K for the leading four scales, so it is
-//    an integer of at most 2^24 times a power of two and exact in FP32 (the lower scales, 2^-32
-//    and below, may round at 2^-24 of themselves).  Every accumulator is read out after every
-//    chunk into a per-element float-float (hi, lo) sum.  The optional tail variants keep t+u = 2
-//    .. BANDS in their own accumulators and the rest in a shared tail, where the tensor core
-//    drops the low bits of the smaller products: BANDS = 5 (NC = 48) gives a floor near 2^-43 of
-//    the result, BANDS = 4 (NC = 64) near 2^-38;
+//    the tensor pipe fed at N = 2NC = 80.  Scale s = t+u-2 sums s+1 products per K, so over
+//    1024 / (s+1) stacked-K elements every partial sum is an integer of at most 2^24 times a power
+//    of two and exact in FP32 (scales 0-3; the lower ones, 2^-32 and below, may round at 2^-24 of
+//    themselves).  The accumulators are read out into a per-element float-float (hi, lo) sum
+//    at the ends of chunks of 256: scales 2 and 3 after every chunk, scale 1 after every second, the
+//    others after every fourth, and all at the end of a tile (split_read_mask).  The optional tail
+//    variants keep t+u = 2 .. BANDS in their own accumulators and the rest in a shared tail, read out
+//    after every chunk, where the tensor core drops the low bits of the smaller products: BANDS = 5
+//    (NC = 48) gives a floor near 2^-43 of the result, BANDS = 4 (NC = 64) near 2^-38;
 //  * the epilogue scales by 2^(E_m + F_n - 14) and forms C = alpha*(hi+lo)*scale + beta*C.
 // Pipeline (persistent, one CTA per SM, tiles claimed from a counter in list order and handed on
-// through a small shared-memory queue): warp 0 claims tiles and issues TMA loads (2 to 6 stages,
-// as many as fit shared memory, of S A tiles 128x32 and S B tiles 2NCx32, BF16, 64-byte
-// swizzle), one thread of warp 1 issues the MMAs (M=128, K=16), warps 2-17 read TMEM and convert
-// and store finished tiles while the next tile's MMAs run.  Every mbarrier wait is bounded: on
-// time-out the kernel flags NDSI timeout status, drains what it issued and frees its TMEM.
+// through a small shared-memory queue): warp 0 claims tiles and issues TMA loads of single digit
+// tiles (A: 128 x 64, B: 2NC x 64, BF16, 128-byte swizzle) into two rings, one thread of warp 1 issues
+// the MMAs (M=128, K=16) and gives every tile back as soon as its last product is issued, warps
+// 2-17 read TMEM and convert and store finished tiles while the next tile's MMAs run.  Every mbarrier
+// wait is bounded: on time-out the kernel flags NDSI timeout status, drains what it issued and frees
+// its TMEM.
+//
+// Why rings of digit tiles.  A 64-wide K block of six digits is 156 KB, so whole blocks leave no room
+// for a second one; with 32-wide blocks in two whole stages (64-byte rows) a stage was refilled only
+// after its last product, and the tensor pipe waited for the load latency of 80 KB each time (53-57%
+// active, 25 bytes per clock and SM).  Here the high B digits (with the A digits that meet them) go
+// first and are given back after 2/7 of the block, the A digits one by one, so that every load has
+// most of a block's time (4000 clocks at six digits; a load from L2 takes 2100) to arrive.  What
+// bounds it now is shared memory: a block's products read 360 KB of operands and the loads write
+// 156 KB, 4000 clocks at 128 bytes each against 3360 of tensor work.  Of the rest, 6% is the wait for
+// read-outs (with all six accumulators read every chunk: 20%) and 15% late loads.  Measured against
+// the two-stage form: 3D metallic lattice T = G_RR L_RJ 1435 -> 1557 TFLOP/s issued, Schur update
+// 1131 -> 1324; 3D cubic lattice 803 -> 1003 (Schur).  Tried without gain: a second producer thread
+// for B, L2 prefetches two blocks ahead (3% slower), 256-byte L2 promotion, giving the scales from 3
+// on back before the others.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_runtime.h>
@@ -274,17 +290,18 @@ __device__ __forceinline__ void tmem_wait_ld(uint32_t* r) {
     for (int i = 0; i < N; ++i) asm volatile("" : "+r"(r[i]));
 }
 
-// Bytes of one K-major tile row (the stage's K in BF16) and the matching swizzle.
-constexpr int kRowBytes = kSplitKB * 2;
-constexpr int kK16Steps = kSplitKB / 16;  // K16 MMA steps per stage
-// Shared-memory matrix descriptor: K-major tile of 8-row x kRowBytes swizzle atoms stacked along M
-// (stride 8 rows), descriptor version 1, 32-byte (layout 6) or 64-byte (layout 4) swizzle.
+// Bytes of one K-major tile row (a block's K in BF16): one 128-byte swizzle atom row.
+constexpr int kRowBytes = kSplitStageK * 2;
+constexpr int kK16Steps = kSplitStageK / 16;  // K16 MMA steps per block
+static_assert(kRowBytes == 128, "tiles use the 128-byte swizzle");
+// Shared-memory matrix descriptor: K-major tile of 8-row x 128-byte swizzle atoms stacked along M
+// (stride 8 rows), descriptor version 1, 128-byte swizzle (layout 2).
 __device__ __forceinline__ uint64_t sdesc_sw(uint32_t saddr) {
     uint64_t d = static_cast<uint64_t>((saddr >> 4) & 0x3FFFu);
     d |= static_cast<uint64_t>(1) << 16;
     d |= static_cast<uint64_t>((8 * kRowBytes) >> 4) << 32;
     d |= static_cast<uint64_t>(1) << 46;
-    d |= static_cast<uint64_t>(kRowBytes == 32 ? 6 : 4) << 61;
+    d |= static_cast<uint64_t>(2) << 61;
     return d;
 }
 // Instruction descriptor: D = F32, A = B = BF16, both K-major, M = 128, N = n (multiple of 16).
@@ -301,77 +318,31 @@ __device__ __forceinline__ void ff_add(float& hi, float& lo, float v) {
     lo += e;
 }
 
-// (hi + lo) * 2^e rounded to nearest double, using integer operations only (GB300's FP64 pipe is
-// the scarce unit): both floats become signed integer mantissas at a common exponent, their
-// exact sum (an int64) is rounded to 53 bits and packed with the combined exponent.  Out of the
-// normal double range it falls back to FP64 arithmetic.
-// Out-of-range results (never produced by finite fronts in practice) take the FP64 route in a
-// separate function so that the common path carries no FP64 instructions, even predicated ones.
+// (hi + lo) * 2^e rounded to double (negated when `negate`), FP32 and integer operations only (GB300's
+// FP64 pipe is the scarce unit): the pair is renormalised by a two-sum so that lo lies 24 binary
+// places or more below hi, lo's mantissa is shifted under hi's in a 64-bit integer, and the sum is
+// rounded to 53 bits.  Infinities, NaN and results outside the normal range take the FP64 route in a
+// separate function, so that the common path carries no FP64 instructions, even predicated ones.
 __device__ __noinline__ double ff_to_double_slow(float hi, float lo, int e, bool negate) {
     const double v = ldexp(static_cast<double>(hi) + static_cast<double>(lo), e);
     return negate ? -v : v;
 }
 
 __device__ __forceinline__ double ff_to_double_scaled(float hi, float lo, int e, bool negate = false) {
-    const uint32_t bh = __float_as_uint(hi), bl = __float_as_uint(lo);
-    const int eh = static_cast<int>((bh >> 23) & 0xFF), el = static_cast<int>((bl >> 23) & 0xFF);
-    int64_t mh = eh ? static_cast<int64_t>((bh & 0x7FFFFFu) | 0x800000u) : 0;
-    int64_t ml = el ? static_cast<int64_t>((bl & 0x7FFFFFu) | 0x800000u) : 0;
-    if (bh >> 31) mh = -mh;
-    if (bl >> 31) ml = -ml;
-    int64_t S;
-    int E0;
-    if (ml == 0) {
-        if (mh == 0) return 0.0;
-        S = mh;
-        E0 = eh - 150;
-    } else if (mh == 0) {
-        S = ml;
-        E0 = el - 150;
-    } else {
-        int64_t big = mh, small = ml;
-        int ebig = eh, esmall = el;
-        if (el > eh) {
-            big = ml;
-            small = mh;
-            ebig = el;
-            esmall = eh;
-        }
-        const int d = ebig - esmall;
-        if (d <= 38) {
-            S = (big << d) + small;
-            E0 = esmall - 150;
-        } else {
-            S = (big << 38) + (small >> (d - 38));
-            E0 = ebig - 150 - 38;
-        }
-    }
-    const bool neg = (S < 0) != negate;
-    uint64_t u = static_cast<uint64_t>(S < 0 ? -S : S);
-    if (u == 0) return 0.0;
-    const int nbits = 64 - __clzll(static_cast<long long>(u));
-    int exp2;
-    uint64_t mant;
-    if (nbits > 53) {
-        int sh = nbits - 53;
-        mant = u >> sh;
-        const uint64_t rem = u & ((uint64_t(1) << sh) - 1);
-        const uint64_t half = uint64_t(1) << (sh - 1);
-        if (rem > half || (rem == half && (mant & 1))) ++mant;
-        if (mant >> 53) {
-            mant >>= 1;
-            ++sh;
-        }
-        exp2 = E0 + e + sh + 52;
-    } else {
-        mant = u << (53 - nbits);
-        exp2 = E0 + e - (53 - nbits) + 52;
-    }
-    const int biased = exp2 + 1023;
-    if (biased <= 0 || biased >= 2047) return ff_to_double_slow(hi, lo, e, negate);
-    const uint64_t bits = (static_cast<uint64_t>(neg) << 63) | (static_cast<uint64_t>(biased) << 52) |
-                          (mant & ((uint64_t(1) << 52) - 1));
-    return __longlong_as_double(static_cast<long long>(bits));
+    const float s = hi + lo, bb = s - hi;
+    const float t = (hi - (s - bb)) + (lo - bb);
+    const uint32_t us = __float_as_uint(s), ut = __float_as_uint(t);
+    const int es = static_cast<int>((us >> 23) & 0xFF), et = static_cast<int>((ut >> 23) & 0xFF);
+    const uint64_t ms = static_cast<uint64_t>((us & 0x7FFFFFu) | 0x800000u) << 39;
+    const uint64_t mt = et ? (static_cast<uint64_t>((ut & 0x7FFFFFu) | 0x800000u) << 15) >> min(max(es - et - 24, 0), 63) : 0;
+    const uint64_t r = (us ^ ut) >> 31 ? ms - mt : ms + mt;
+    const int lz = __clzll(static_cast<long long>(r));  // 1 or 2
+    const uint64_t n = r << lz;
+    const int biased = 63 - lz + es - 189 + e + 1023;
+    if (es == 0 || es == 255 || biased <= 0 || biased >= 2046)
+        return es == 0 && (us << 1) == 0 ? 0.0 : ff_to_double_slow(hi, lo, e, negate);
+    const uint64_t bits = (static_cast<uint64_t>(biased - 1) << 52) + (n >> 11) + ((n >> 10) & 1);
+    return __longlong_as_double(static_cast<long long>(bits | static_cast<uint64_t>((us >> 31) ^ (negate ? 1u : 0u)) << 63));
 }
 
 // ----------------------------------------------------------------------------- slicing -----
@@ -792,51 +763,48 @@ template <int CW>
 constexpr bool kEpiDoubleBuffer = CW <= 12;
 
 template <int NC>
-__host__ __device__ constexpr int tile_bytes_b() { return 2 * NC * kRowBytes; }  // 2NC rows x kRowBytes
-template <int S, int NC>
-__host__ __device__ constexpr int stage_bytes() { return S * (kTileBytes + tile_bytes_b<NC>()); }
-// barriers (256 B), the tile's row / column exponents (768 B) and up to 1 KB lost to aligning the
-// tiles to 1024 bytes
-constexpr int kSplitSmemExtra = 256 + 768 + 1024;
-constexpr int kSplitMaxStages = 6;
-// Pipeline depth: as many stages (2..6) as fit the 227 KB of shared memory a CTA may use.
-template <int S, int NC>
-__host__ __device__ constexpr int split_stages() {
-    return (227 * 1024 - kSplitSmemExtra) / stage_bytes<S, NC>() >= kSplitMaxStages
-               ? kSplitMaxStages
-               : ((227 * 1024 - kSplitSmemExtra) / stage_bytes<S, NC>() < 2
-                      ? 2
-                      : (227 * 1024 - kSplitSmemExtra) / stage_bytes<S, NC>());
-}
-template <int S, int NC>
-__host__ __device__ constexpr int split_smem_bytes() {
-    return split_stages<S, NC>() * stage_bytes<S, NC>() + kSplitSmemExtra;
-}
+__host__ __device__ constexpr int tile_bytes_b() { return 2 * NC * kRowBytes; }  // 2NC rows x 128 bytes
 // Per-scale mode: one accumulator per t+u (any tile width other than the two tail variants).
 template <int NC>
 __host__ __device__ constexpr bool split_exact_mode() { return NC != kSplitBNc && NC != kSplitBNc5; }
-
-// The MMAs of one A digit t in per-scale mode: A_t times the stage's B digits 0 .. S-1-t, which
-// are consecutive rows of one K-major block, land in accumulator columns t*NB .. S*NB, i.e. the
-// product with B_u in the accumulator of scale t+u.  Issued in pieces of at most 256 rows.
-template <int S, int NB, int T, int R0>
-__device__ __forceinline__ void issue_digit(uint32_t tmem, uint64_t da, uint64_t db0, int ks, uint32_t acc) {
-    constexpr int rows = (S - T) * NB;
-    if constexpr (R0 < rows) {
-        constexpr int n = rows - R0 < 256 ? rows - R0 : 256;
-        const uint64_t db = db0 + static_cast<uint64_t>((R0 * kRowBytes + ks * 32) >> 4);
-        umma_bf16(tmem + T * NB + R0, da, db, idesc_bf16(n), acc);
-        issue_digit<S, NB, T, R0 + 256>(tmem, da, db0, ks, acc);
-    }
+// barriers (512 B), the tile's row / column exponents (768 B) and up to 1 KB lost to aligning the
+// tiles to 1024 bytes
+constexpr int kSplitSmemExtra = 512 + 768 + 1024;
+constexpr int kSplitSmemMax = 227 * 1024;
+// Rings.  B digits move in groups of consecutive rows that one MMA (N <= 256) covers: in per-scale
+// mode two groups per block, the low digits [0, G) and the high ones [G, S), in a ring of three;
+// in the tail variants single digits.  A digits move singly, eight slots (seven beside the widest B).
+template <int S, int NC>
+struct SplitRing {
+    static constexpr bool EXACT = split_exact_mode<NC>();
+    static constexpr int G = EXACT ? 256 / (2 * NC) : 1;            // B digits per group
+    static constexpr int PER = EXACT ? 2 : S;                       // groups per block
+    static constexpr int GROUP = G * tile_bytes_b<NC>();
+    static constexpr int NA = NC == kSplitBNc ? 7 : 8;              // A slots
+    static constexpr int FIT = (kSplitSmemMax - kSplitSmemExtra - NA * kTileBytes) / GROUP;
+    static constexpr int NG = EXACT ? 3 : (FIT < 9 ? FIT : 9);      // B group slots
+    static constexpr int BYTES = NA * kTileBytes + NG * GROUP;
+    static_assert(NG <= FIT && NG > PER - 1 && G < S, "rings exceed shared memory");
+};
+template <int S, int NC>
+__host__ __device__ constexpr int split_smem_bytes() {
+    return SplitRing<S, NC>::BYTES + kSplitSmemExtra;
 }
-template <int S, int NB, int KT, int T>
-__device__ __forceinline__ void issue_digits(uint32_t tmem, uint64_t da0, uint64_t db0, int ks, uint32_t fresh) {
-    if constexpr (T < S) {
-        const uint64_t da = da0 + static_cast<uint64_t>((T * KT + ks * 32) >> 4);
-        // the first digit writes every accumulator: it starts the chunk's sums on its first K16
-        issue_digit<S, NB, T, 0>(tmem, da, db0, ks, (T == 0 && ks == 0) ? fresh : 1u);
-        issue_digits<S, NB, KT, T + 1>(tmem, da0, db0, ks, fresh);
-    }
+
+// Accumulators read out after chunk k of a tile (bit s: scale t+u = s+2), beside every one after the
+// last chunk.  Scale s sums s+1 products of at most 2^14 per K element, so its sums stay below 2^24
+// and exact for 1024/(s+1) elements: scales 2 and 3 are read every chunk of 256, scale 1 every second
+// and scale 0 every fourth.  The scales from 4 on (2^-32 and below of the product) may round at 2^-24
+// of themselves either way and are read every fourth chunk.
+template <int S>
+__host__ __device__ constexpr uint32_t split_read_mask(int k, bool last) {
+    return last || (k & 3) == 3 ? (1u << S) - 1 : (k & 1) ? 0xEu : 0xCu;
+}
+
+// Read-out order of the accumulators: the first two and the first three are those of the masks above.
+template <bool EXACT>
+__host__ __device__ constexpr int split_read_order(int i) {
+    return !EXACT ? i : i == 0 ? 2 : i == 1 ? 3 : i == 2 ? 1 : i == 3 ? 0 : i;
 }
 
 template <int S, int NC>
@@ -844,21 +812,20 @@ __global__ void __launch_bounds__(kThreads, 1)
     k_gemm_split(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmArgs p) {
     constexpr bool EXACT = split_exact_mode<NC>();
     // TMEM accumulators: one per scale (EXACT), else four or five with a tail; BANDS x 2NC <= 512
-    constexpr int BANDS = EXACT ? S : (NC == kSplitBNc ? 4 : 5);
+    constexpr int BANDS = EXACT || S < 5 ? S : (NC == kSplitBNc ? 4 : 5);  // four slices: four scales in all
     constexpr int NB = 2 * NC;                       // accumulator columns per band (Re | Im)
     constexpr int CW = NC / 4;                       // complex columns per epilogue warp
     constexpr int kTileB = tile_bytes_b<NC>();
-    constexpr int kStage = stage_bytes<S, NC>();
-    constexpr int STAGES = split_stages<S, NC>();
-    constexpr uint32_t kId = idesc_bf16(NB);
+    using Ring = SplitRing<S, NC>;
+    constexpr int NA = Ring::NA, NG = Ring::NG, G = Ring::G, PER = Ring::PER;
     static_assert(BANDS * NB <= 512, "accumulators exceed TMEM");
     static_assert(CW % 2 == 0, "epilogue column groups read TMEM in pairs of columns");
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * kStage);
-    uint64_t* full = bars;                 // [STAGES]
-    uint64_t* empty = bars + kSplitMaxStages;  // [STAGES]
-    uint64_t* chunk_full = bars + 2 * kSplitMaxStages;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Ring::BYTES);
+    uint64_t *a_full = bars, *a_empty = bars + NA;                    // [NA] A digit tiles
+    uint64_t *b_full = bars + 2 * NA, *b_empty = b_full + NG;         // [NG] B digit groups
+    uint64_t* chunk_full = b_empty + NG;
     uint64_t* tmem_free = chunk_full + 1;
     uint64_t* mma_done = chunk_full + 2;
     uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(chunk_full + 3);
@@ -868,8 +835,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint64_t* tq_empty = tq_full + kTileQueue;  // [kTileQueue] read by the MMA thread and the epilogue
     volatile int64_t* tq = reinterpret_cast<volatile int64_t*>(tq_empty + kTileQueue);  // [kTileQueue]
     volatile int64_t* epi_w = tq + kTileQueue;  // the epilogue's current tile, broadcast
-    static_assert(2 * kSplitMaxStages + 5 + 3 * kTileQueue + 1 <= 32, "barriers overflow their 256 bytes");
-    int* sm_ea = reinterpret_cast<int*>(bars + 32);  // [128] exponents of the current tile's rows
+    static_assert(2 * NA + 2 * NG + 5 + 3 * kTileQueue + 1 <= 64, "barriers overflow their 512 bytes");
+    int* sm_ea = reinterpret_cast<int*>(bars + 64);  // [128] exponents of the current tile's rows
     int* sm_eb = sm_ea + 128;                         // [64] exponents of its complex columns
 
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -882,14 +849,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int64_t n_work = p.tcount * p.np;
     int* claim = p.status + 2;  // [0] items claimed beyond the first wave, [1] CTAs finished
     auto tile_of = [&](int64_t w) { return p.tiles[p.tfirst + w % p.tcount]; };
-    auto nkb_of = [&](const GemmTile& t) { return 2 * p.sitems[p.ifirst + t.item].Kpad / kSplitKB; };
+    auto nkb_of = [&](const GemmTile& t) { return 2 * p.sitems[p.ifirst + t.item].Kpad / kSplitStageK; };
 
     if (threadIdx.x == 0) {
 #pragma unroll
-        for (int st = 0; st < STAGES; ++st) {
-            mbar_init(&full[st], 1);
-            mbar_init(&empty[st], 1);
-        }
+        for (int i = 0; i < 2 * (NA + NG); ++i) mbar_init(&bars[i], 1);
         mbar_init(chunk_full, 1);
         mbar_init(tmem_free, kEpiWarps);
         mbar_init(mma_done, 1);
@@ -905,14 +869,17 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_holder;
-    auto a_tile = [&](int stage, int t) { return smem + stage * kStage + t * kTileBytes; };
-    auto b_tile = [&](int stage, int u) { return smem + stage * kStage + S * kTileBytes + u * kTileB; };
+    // ring slots: item i of a ring sits in slot i % size, its (i / size)-th use (the phase parity)
+    uint8_t* b_ring = smem + NA * kTileBytes;
 
     if (warp == 0) {
         if (lane == 0) {
-            // producer: one ring of STAGES stages across all of this CTA's tiles
-            int64_t g = 0;      // K-blocks issued so far (all tiles)
-            int64_t armed = 0;
+            // producer: both rings run on across all of this CTA's tiles, in the order the MMA thread
+            // needs them; ia, ib count the A tiles and B groups armed so far
+            int64_t ia = 0, ib = 0;
+            auto slot_free = [&](uint64_t* empty, int64_t i, int n) {
+                return i < n || mbar_wait(&empty[i % n], static_cast<uint32_t>(((i / n) - 1) & 1), abort);
+            };
             for (int64_t jt = 0;; ++jt) {
                 const int slot = static_cast<int>(jt % kTileQueue);
                 if (jt >= kTileQueue &&
@@ -930,35 +897,47 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int yA0 = static_cast<int>(pole * p.rowsA + si.rowA + tile.m0);
                 const int yB0 = static_cast<int>(pole * p.rowsB + si.rowB + (tile.n0 / NC) * NB);
                 bool ok = true;
-                for (int kb = 0; kb < nkb; ++kb, ++g) {
-                    const int stage = static_cast<int>(g % STAGES);
-                    if (g >= STAGES &&
-                        !mbar_wait(&empty[stage], static_cast<uint32_t>(((g / STAGES) - 1) & 1), abort)) {
-                        ok = false;
-                        break;
+                for (int kb = 0; kb < nkb && ok; ++kb) {
+                    const int x = kb * kSplitStageK;
+                    auto load_a = [&](int t) {
+                        if (!ok || !(ok = slot_free(a_empty, ia, NA))) return;
+                        const int sl = static_cast<int>(ia++ % NA);
+                        mbar_expect_tx(&a_full[sl], kTileBytes);
+                        tma_load_2d(smem + sl * kTileBytes, &tmA, x, yA0 + t * si.Mpad, &a_full[sl]);
+                    };
+                    auto load_b = [&](int u0, int u1) {  // digits u0 .. u1-1 into consecutive rows of one group
+                        if (!ok || !(ok = slot_free(b_empty, ib, NG))) return;
+                        const int sl = static_cast<int>(ib++ % NG);
+                        mbar_expect_tx(&b_full[sl], (u1 - u0) * kTileB);
+                        for (int u = u0; u < u1; ++u)
+                            tma_load_2d(b_ring + sl * Ring::GROUP + (u - u0) * kTileB, &tmB, x, yB0 + u * 2 * si.Npad,
+                                        &b_full[sl]);
+                    };
+                    if constexpr (EXACT) {
+                        load_b(G, S);                                    // high digits, needed first
+                        for (int t = 0; t < S - G; ++t) load_a(t);
+                        load_b(0, G);
+                        for (int t = S - G; t < S; ++t) load_a(t);
+                    } else {
+                        for (int u = S - 1; u >= 0; --u) load_b(u, u + 1);
+                        for (int t = 0; t < S; ++t) load_a(t);
                     }
-                    mbar_expect_tx(&full[stage], kStage);
-#pragma unroll
-                    for (int t = 0; t < S; ++t)
-                        tma_load_2d(a_tile(stage, t), &tmA, kb * kSplitKB, yA0 + t * si.Mpad, &full[stage]);
-#pragma unroll
-                    for (int u = 0; u < S; ++u)
-                        tma_load_2d(b_tile(stage, u), &tmB, kb * kSplitKB, yB0 + u * 2 * si.Npad, &full[stage]);
-                    armed = g + 1;
                 }
                 if (!ok) break;
             }
             if (*abort) {
-                // drain: wait for the last (up to STAGES) armed stages' copies to land
-                for (int64_t k = armed > STAGES ? armed - STAGES : 0; k < armed; ++k)
-                    mbar_wait_drain(&full[k % STAGES], static_cast<uint32_t>((k / STAGES) & 1));
+                // drain: wait for the copies of the last armed slots of both rings to land
+                for (int64_t i = ia > NA ? ia - NA : 0; i < ia; ++i)
+                    mbar_wait_drain(&a_full[i % NA], static_cast<uint32_t>((i / NA) & 1));
+                for (int64_t i = ib > NG ? ib - NG : 0; i < ib; ++i)
+                    mbar_wait_drain(&b_full[i % NG], static_cast<uint32_t>((i / NG) & 1));
             }
         }
     } else if (warp == 1) {
         if (lane == 0) {
             // MMA issue: chunks are numbered across tiles; chunk c > 0 starts once the epilogue
             // has read chunk c - 1 out of TMEM (which may belong to the previous tile)
-            int64_t g = 0, c = 0;
+            int64_t ia = 0, ib = 0, c = 0;  // A tiles and B groups consumed, chunks started
             bool ok = true;
             for (int64_t jt = 0; ok; ++jt) {
                 const int slot = static_cast<int>(jt % kTileQueue);
@@ -967,67 +946,105 @@ __global__ void __launch_bounds__(kThreads, 1)
                 mbar_arrive(&tq_empty[slot]);
                 if (w < 0) break;
                 const int nkb = nkb_of(tile_of(w));
-                for (int kb = 0; kb < nkb; ++kb, ++g) {
-                    const int stage = static_cast<int>(g % STAGES);
-                    if (!mbar_wait(&full[stage], static_cast<uint32_t>((g / STAGES) & 1), abort)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
+                uint32_t keep = 0;  // scales whose accumulators hold sums of earlier chunks of the tile
+                for (int kb = 0; kb < nkb && ok; ++kb) {
                     const bool first_in_chunk = (kb % kSplitChunkKB) == 0;
                     if (first_in_chunk && c > 0) {
-                        if (!mbar_wait(tmem_free, static_cast<uint32_t>((c - 1) & 1), abort)) {
-                            ok = false;
-                            break;
-                        }
-                        tc_fence_after();
+                        if (!(ok = mbar_wait(tmem_free, static_cast<uint32_t>((c - 1) & 1), abort))) break;
                     }
-                    // Descriptors of this stage's slice tiles: the start-address field is the low
-                    // 14 bits (address >> 4), so tile t and K16 half ks are compile-time offsets
-                    // from the stage's first tile.  The loops unroll completely (S is a template
-                    // parameter), leaving one 64-bit add and one tcgen05.mma per instruction.
-                    const uint64_t da0 = sdesc_sw(smem_u32(a_tile(stage, 0)));
-                    const uint64_t db0 = sdesc_sw(smem_u32(b_tile(stage, 0)));
-                    const uint32_t fresh = first_in_chunk ? 0u : 1u;
+                    // Descriptors: the start-address field is the low 14 bits (address >> 4), so digit
+                    // tiles and K16 steps are offsets from a slot's descriptor.  The loops unroll
+                    // completely (S is a template parameter).
+                    uint64_t da[S];
+                    auto wait_a = [&](int t) {
+                        const int64_t i = ia + t;
+                        ok = ok && mbar_wait(&a_full[i % NA], static_cast<uint32_t>((i / NA) & 1), abort);
+                        da[t] = sdesc_sw(smem_u32(smem + (i % NA) * kTileBytes));
+                    };
+                    auto free_a = [&](int t) { umma_commit(&a_empty[(ia + t) % NA]); };
+                    auto wait_b = [&](int j) {  // j-th group of this block
+                        const int64_t i = ib + j;
+                        ok = ok && mbar_wait(&b_full[i % NG], static_cast<uint32_t>((i / NG) & 1), abort);
+                        return sdesc_sw(smem_u32(b_ring + (i % NG) * Ring::GROUP));
+                    };
                     if constexpr (EXACT) {
+                        // A_t times digits u0 .. u0+n-1 of a group: one MMA per K16 step into the
+                        // accumulators of scales t+u0 .. t+u0+n-1; the first products of a chunk go
+                        // scale by scale, each starting or continuing its own sum
+                        auto products = [&](int t, int u0, int n, uint64_t db) {
+                            const uint32_t d = tmem + (t + u0) * NB;
 #pragma unroll
-                        for (int ks = 0; ks < kK16Steps; ++ks) issue_digits<S, NB, kTileBytes, 0>(tmem, da0, db0, ks, fresh);
-                    } else {
-                        // tail band BANDS-1: slice pairs with t+u >= BANDS+1 (1-based), read out per
-                        // chunk like the others
+                            for (int ks = 0; ks < kK16Steps; ++ks) {
+                                const uint64_t a = da[t] + static_cast<uint64_t>((ks * 32) >> 4);
+                                const uint64_t b = db + static_cast<uint64_t>((ks * 32) >> 4);
+                                if (t == 0 && ks == 0 && first_in_chunk) {
 #pragma unroll
-                        for (int t = 0; t < S; ++t)
-#pragma unroll
-                            for (int u = 0; u < S; ++u) {
-                                if (t + u > S - 1 || t + u < BANDS - 1) continue;
-                                const bool lead = (t + u == BANDS - 1) && t == 0;  // first tail product of a K-block
-#pragma unroll
-                                for (int ks = 0; ks < kK16Steps; ++ks) {
-                                    const uint64_t da = da0 + static_cast<uint64_t>((t * kTileBytes + ks * 32) >> 4);
-                                    const uint64_t db = db0 + static_cast<uint64_t>((u * kTileB + ks * 32) >> 4);
-                                    umma_bf16(tmem + (BANDS - 1) * NB, da, db, kId, (lead && ks == 0) ? fresh : 1u);
+                                    for (int u = 0; u < G; ++u)
+                                        if (u < n)
+                                            umma_bf16(d + u * NB, a, b + static_cast<uint64_t>((u * kTileB) >> 4),
+                                                      idesc_bf16(NB), (keep >> (u0 + u)) & 1u);
+                                } else {
+                                    umma_bf16(d, a, b, idesc_bf16(static_cast<uint32_t>(n * NB)), 1u);
                                 }
                             }
-                        // exact bands 0..BANDS-2: t+u = 2 .. BANDS (1-based), one scale each
+                        };
+                        const uint64_t bh = wait_b(0);
 #pragma unroll
-                        for (int band = 0; band < BANDS - 1; ++band) {
-#pragma unroll
-                            for (int t = 0; t < S; ++t) {
-                                const int u = band - t;
-                                if (u < 0 || u >= S) continue;
-#pragma unroll
-                                for (int ks = 0; ks < kK16Steps; ++ks) {
-                                    const uint64_t da = da0 + static_cast<uint64_t>((t * kTileBytes + ks * 32) >> 4);
-                                    const uint64_t db = db0 + static_cast<uint64_t>((u * kTileB + ks * 32) >> 4);
-                                    umma_bf16(tmem + band * NB, da, db, kId, (t == 0 && ks == 0) ? fresh : 1u);
-                                }
-                            }
+                        for (int t = 0; t < S - G; ++t) {
+                            wait_a(t);
+                            if (!ok) break;
+                            tc_fence_after();
+                            products(t, G, S - G - t, bh);
                         }
+                        if (!ok) break;
+                        umma_commit(&b_empty[ib % NG]);
+                        const uint64_t bl = wait_b(1);
+#pragma unroll
+                        for (int t = 0; t < S; ++t) {
+                            if (t >= S - G) wait_a(t);
+                            if (!ok) break;
+                            tc_fence_after();
+                            products(t, 0, S - t < G ? S - t : G, bl);
+                            free_a(t);
+                        }
+                        if (!ok) break;
+                        umma_commit(&b_empty[(ib + 1) % NG]);
+                    } else {
+                        // bands 0..BANDS-2 hold one scale each, band BANDS-1 the rest; digit u is group
+                        // S-1-u of the block and free once A_{S-1-u} has met it
+                        uint64_t db[S];
+#pragma unroll
+                        for (int u = S - 1; u >= 0; --u) db[u] = wait_b(S - 1 - u);
+#pragma unroll
+                        for (int t = 0; t < S; ++t) {
+                            wait_a(t);
+                            if (!ok) break;
+                            tc_fence_after();
+#pragma unroll
+                            for (int u = S - 1; u >= 0; --u) {
+                                if (t + u > S - 1) continue;
+                                constexpr int last = BANDS - 1;
+                                const int band = t + u < last ? t + u : last;
+                                // the first product into a band: t == 0, and for the tail the first u
+                                const bool lead = t == 0 && (t + u < last || u == S - 1);
+#pragma unroll
+                                for (int ks = 0; ks < kK16Steps; ++ks)
+                                    umma_bf16(tmem + band * NB, da[t] + static_cast<uint64_t>((ks * 32) >> 4),
+                                              db[u] + static_cast<uint64_t>((ks * 32) >> 4), idesc_bf16(NB),
+                                              lead && ks == 0 && first_in_chunk ? 0u : 1u);
+                            }
+                            free_a(t);
+                            umma_commit(&b_empty[(ib + t) % NG]);
+                        }
+                        if (!ok) break;
                     }
-                    umma_commit(&empty[stage]);
-                    if ((kb % kSplitChunkKB) == kSplitChunkKB - 1 || kb == nkb - 1) {
+                    ia += S;
+                    ib += PER;
+                    const bool last_kb = kb == nkb - 1;
+                    if ((kb % kSplitChunkKB) == kSplitChunkKB - 1 || last_kb) {
                         umma_commit(chunk_full);
                         ++c;
+                        if constexpr (EXACT) keep = ((1u << S) - 1) & ~split_read_mask<S>(kb / kSplitChunkKB, last_kb);
                     }
                 }
             }
@@ -1099,9 +1116,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                     break;
                 }
                 tc_fence_after();
-                // A band's Re and Im columns are requested together and awaited once; with two
-                // buffers the next band's loads are in flight while this band's sums run.  TMEM goes
-                // back to the MMA warp as soon as the last band is in registers.
+                // The accumulators due after this chunk, in the order 2, 3, 1, 0, 4, 5, .. (so that the
+                // ones due more often come first) or all bands of the tail variants.  A band's Re and
+                // Im columns are requested together and awaited once, two bands ahead of the sums;
+                // TMEM goes back to the MMA warp as soon as the last band is in registers: before any
+                // sum when two are due.
                 auto load_band = [&](int band, uint32_t* r) {
 #pragma unroll
                     for (int part = 0; part < 2; ++part)  // Re columns, then the matching Im columns
@@ -1114,24 +1133,50 @@ __global__ void __launch_bounds__(kThreads, 1)
                     __syncwarp();
                     if (lane == 0) mbar_arrive(tmem_free);
                 };
-                auto sum_band = [&](const uint32_t* r) {
+                // Scales from 3 on lie below 2^-24 of the product, where the low part's own rounding is:
+                // they join it by one addition; the others enter the pair by a two-sum.
+                auto sum_band = [&](auto band, const uint32_t* r) {
 #pragma unroll
-                    for (int i = 0; i < 2 * CW; ++i) ff_add(hi[i], lo[i], __uint_as_float(r[i]));
+                    for (int i = 0; i < 2 * CW; ++i) {
+                        if constexpr (EXACT && decltype(band)::value >= 3) lo[i] += __uint_as_float(r[i]);
+                        else ff_add(hi[i], lo[i], __uint_as_float(r[i]));
+                    }
                 };
                 (void)load_band;
                 (void)sum_band;
                 if constexpr (kEpiDoubleBuffer<CW>) {
-                    uint32_t r[2][2 * CW];
-                    load_band(0, r[0]);
-                    tmem_wait_ld<2 * CW>(r[0]);
-#pragma unroll
-                    for (int band = 0; band < BANDS; ++band) {
-                        if (band + 1 < BANDS) load_band(band + 1, r[(band + 1) & 1]);
-                        sum_band(r[band & 1]);
-                        if (band + 1 < BANDS) tmem_wait_ld<2 * CW>(r[(band + 1) & 1]);
-                        if (band + 1 == BANDS - 1) release();
+                    auto read_out = [&](auto count) {
+                        constexpr int N = decltype(count)::value;
+                        uint32_t r[2][2 * CW];
+                        auto step = [&](auto self, auto idx) {
+                            constexpr int I = decltype(idx)::value;
+                            if constexpr (I < N) {
+                                // r[I & 1] holds band I; its successor but one reuses the registers
+                                if constexpr (I > 1) {
+                                    tmem_wait_ld<2 * CW>(r[I & 1]);
+                                    if constexpr (I == N - 1) release();
+                                }
+                                sum_band(std::integral_constant<int, split_read_order<EXACT>(I)>{}, r[I & 1]);
+                                if constexpr (I + 2 < N) load_band(split_read_order<EXACT>(I + 2), r[I & 1]);
+                                self(self, std::integral_constant<int, I + 1>{});
+                            }
+                        };
+                        load_band(split_read_order<EXACT>(0), r[0]);
+                        load_band(split_read_order<EXACT>(1), r[1]);
+                        tmem_wait_ld<2 * CW>(r[0]);
+                        tmem_wait_ld<2 * CW>(r[1]);
+                        if constexpr (N == 2) release();
+                        step(step, std::integral_constant<int, 0>{});
+                    };
+                    static_assert(BANDS > 2, "two bands are loaded at a time");
+                    if constexpr (EXACT) {
+                        const int due = __popc(split_read_mask<S>(k, k == nchunks - 1));
+                        if (due == 2) read_out(std::integral_constant<int, 2>{});
+                        else if (due == 3) read_out(std::integral_constant<int, 3>{});
+                        else read_out(std::integral_constant<int, BANDS>{});
+                    } else {
+                        read_out(std::integral_constant<int, BANDS>{});
                     }
-                    if constexpr (BANDS == 1) release();
                 } else {
                     // wide column groups: one part (Re or Im columns) at a time
 #pragma unroll
@@ -1159,21 +1204,34 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int m = tile.m0 + r;
             if (m < it.M) {
                 const int ea = sm_ea[r] - 14;
+                auto live = [&](int j) {
+                    const int n = tile.n0 + cg * CW + j;
+                    return n < it.N && !(p.lower && n > m);
+                };
+                auto at = [&](int j) { return Cp + m + static_cast<int64_t>(tile.n0 + cg * CW + j) * it.ldc; };
+                // C is requested a few columns ahead of the conversions, so that their loads overlap
+                constexpr int AHEAD = CW <= 10 ? 5 : CW <= 12 ? 3 : 2;
+                double2 old[AHEAD];
 #pragma unroll
-                for (int j = 0; j < CW; ++j) {
-                    const int jc = cg * CW + j;
-                    const int n = tile.n0 + jc;
-                    if (n >= it.N || (p.lower && n > m)) continue;
-                    double2* dst = Cp + m + static_cast<int64_t>(n) * it.ldc;
-                    const int e = ea + sm_eb[jc];
-                    double re = ff_to_double_scaled(hi[j], lo[j], e, neg_alpha);
-                    double im = ff_to_double_scaled(hi[CW + j], lo[CW + j], e, neg_alpha);
-                    if (add_c) {
-                        const double2 old = *dst;
-                        re += old.x;
-                        im += old.y;
+                for (int j0 = 0; j0 < CW; j0 += AHEAD) {
+#pragma unroll
+                    for (int u = 0; u < AHEAD; ++u) {
+                        old[u] = make_double2(0.0, 0.0);
+                        if (add_c && j0 + u < CW && live(j0 + u)) old[u] = *at(j0 + u);
                     }
-                    *dst = make_double2(re, im);
+#pragma unroll
+                    for (int u = 0; u < AHEAD; ++u) {
+                        const int j = j0 + u;
+                        if (j >= CW || !live(j)) continue;
+                        const int e = ea + sm_eb[cg * CW + j];
+                        double re = ff_to_double_scaled(hi[j], lo[j], e, neg_alpha);
+                        double im = ff_to_double_scaled(hi[CW + j], lo[CW + j], e, neg_alpha);
+                        if (add_c) {
+                            re += old[u].x;
+                            im += old[u].y;
+                        }
+                        *at(j) = make_double2(re, im);
+                    }
                 }
             }
         }
@@ -1211,7 +1269,8 @@ template <int S>
 cudaError_t set_attrs() {
     cudaError_t e = set_gemm_attr<S, kSplitBNc>();
     if (e == cudaSuccess) e = set_gemm_attr<S, kSplitBNc5>();
-    if (e == cudaSuccess) e = set_gemm_attr<S, kSplitBNcX7>();
+    if constexpr (S >= 6)  // seven slices, and the far poles of a seven-slice plan
+        if (e == cudaSuccess) e = set_gemm_attr<S, kSplitBNcX7>();
     if constexpr (S <= 6)
         if (e == cudaSuccess) e = set_gemm_attr<S, kSplitBNcX>();
     if (e != cudaSuccess) return e;
@@ -1252,11 +1311,11 @@ void split_free(SplitBuffers& B) {
 static cudaError_t encode(CUtensorMap* map, void* base, int64_t cols, int64_t rows, int box_rows) {
     cuuint64_t dims[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
     cuuint64_t strides[1] = {static_cast<cuuint64_t>(cols * 2)};
-    cuuint32_t box[2] = {static_cast<cuuint32_t>(kSplitKB), static_cast<cuuint32_t>(box_rows)};
+    cuuint32_t box[2] = {static_cast<cuuint32_t>(kSplitStageK), static_cast<cuuint32_t>(box_rows)};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, estr,
                           CU_TENSOR_MAP_INTERLEAVE_NONE,
-                          kRowBytes == 32 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_64B,
+                          CU_TENSOR_MAP_SWIZZLE_128B,
                           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
@@ -1337,7 +1396,9 @@ static cudaError_t run_mma(const Launch& l, int step_index, const GemmItem* item
     switch (step.nc) {
         case kSplitBNc: return go(std::integral_constant<int, kSplitBNc>{});
         case kSplitBNc5: return go(std::integral_constant<int, kSplitBNc5>{});
-        case kSplitBNcX7: return go(std::integral_constant<int, kSplitBNcX7>{});
+        case kSplitBNcX7:
+            if constexpr (S >= 6) return go(std::integral_constant<int, kSplitBNcX7>{});
+            return cudaErrorInvalidValue;
         case kSplitBNcX:
             if constexpr (S <= 6) return go(std::integral_constant<int, kSplitBNcX>{});
             return cudaErrorInvalidValue;

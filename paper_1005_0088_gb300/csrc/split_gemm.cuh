@@ -27,16 +27,9 @@ constexpr int split_nc(int slices, int bands) {
 constexpr int kSplitSliceRows = 32;  // operand rows per slicing block (two-pass slicer)
 constexpr int kSplitSlice1Smem = 72 * 1024;       // one-pass slicer budget, 4..32 rows per block
 constexpr int kSplitSlice1SmemWide = 200 * 1024;  // budget for very long rows, 1 or 2 rows per block
-// Stacked K per pipeline stage: 32 BF16 (64-byte rows, 64-byte swizzle, two K16 MMA steps per
-// digit).  16 (32-byte rows, 32-byte swizzle) fits five stages at six slices instead of two, but
-// its half-size row requests loaded L1 and L2 far more and the 3D metallic sweep ran 9% slower.
-#ifdef NDSI_SPLIT_KB
-constexpr int kSplitKB = NDSI_SPLIT_KB;
-#else
-constexpr int kSplitKB = 32;
-#endif
-static_assert(kSplitKB == 16 || kSplitKB == 32, "stage K must be 16 or 32");
-constexpr int kSplitChunkKB = 256 / kSplitKB;   // stages per exact chunk (256 stacked-K elements)
+constexpr int kSplitKB = 32;       // complex K padding: the stacked K (2 Kpad) is a multiple of kSplitStageK
+constexpr int kSplitStageK = 64;   // stacked K per pipeline block: 64 BF16 (128-byte rows, 128-byte swizzle)
+constexpr int kSplitChunkKB = 256 / kSplitStageK;  // blocks per exact chunk (256 stacked-K elements)
 constexpr int kSplitMaxSlices = 7;
 // Bytes of one operand's slices a tile group may keep in L2 while the other operand streams
 // (a third of GB300's 126 MB L2), and the tiles the persistent GEMM runs at one time (one CTA on

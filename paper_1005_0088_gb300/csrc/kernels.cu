@@ -9,6 +9,7 @@
 #include <cstdint>
 #include <cstring>
 
+#include "fixed_point.cuh"
 #include "kernels.cuh"
 
 namespace ndsi {
@@ -274,92 +275,6 @@ __global__ void __launch_bounds__(32) k_diaginv_sweep(const DiagItem* __restrict
         if (i < nb && k < nb) A[i + static_cast<int64_t>(k) * ld] = make_double2(-a[s].x, -a[s].y);
     }
 }
-
-// ---------------------------------------------------------------------------------------------
-// Fixed-point products.  GB300 issues one warp-wide FP64 instruction per SM every 16-19 clocks (1.7-2
-// lanes a clock; 64 clocks per sub-partition) but 59 lanes a clock of 32 x 32 + 64-bit integer
-// multiply-adds (both measured), so products of complex matrices are formed in 57-bit fixed point:
-// over at most 32 inner indices every row of op(A) and column of op(B) is scaled by a power of two
-// and cut to x = (h 2^29 + l) 2^(E - 57), |h| <= 2^28, -2^28 <= l < 2^28.  Twelve integer
-// multiply-adds per complex product accumulate the h h and h l + l h sums exactly in 64 bits
-// (|sum| <= 2^62 and 2^63 over 32 terms; l l, below 2^-57 of the row times column maximum, is
-// dropped), and the sum is rounded once to FP64.  The error of an output is about 2^-57 of (row
-// maximum) x (column maximum) per term plus that one rounding, against one FP64 rounding per term
-// and accumulator of a DFMA loop.  The basis functions are brought to a common scale beforehand
-// (launch_basis_scale), so that a row's maximum speaks for the row.
-// Rows or columns holding an infinity or NaN give NaN.
-constexpr int kFixK = 32;          // inner indices per exact integer sum
-constexpr int kFixNonFinite = 1 << 20;  // row exponent of a row holding an infinity or NaN
-
-// Digits of x at row exponent field `emax` (x == 0 or its exponent field <= emax): F = x 2^(57 - E) cut
-// towards zero.
-__device__ __forceinline__ void fix_digits(double x, int emax, int& h, int& l) {
-    const int64_t b = __double_as_longlong(x);
-    const int ex = static_cast<int>((b >> 52) & 0x7FF);
-    const uint64_t m = (static_cast<uint64_t>(b) << 10 & 0x3FFFFFFFFFFFFFFFull) | 0x4000000000000000ull;  // 1.f at bit 62
-    const int sh = ex ? min(6 + emax - ex, 63) : 63;
-    int64_t f = static_cast<int64_t>(m >> sh);
-    f = b < 0 ? -f : f;
-    l = static_cast<int>(static_cast<uint32_t>(f) << 3) >> 3;
-    h = static_cast<int>((f - l) >> 29);
-}
-
-__device__ __noinline__ double fix_to_double_slow(int64_t t, uint32_t rem, int e) {
-    if (e >= kFixNonFinite / 2) return __longlong_as_double(0x7FF8000000000000ll);
-    return ldexp(ldexp(static_cast<double>(t), 29) + static_cast<double>(rem), e + 29);
-}
-// (hh 2^58 + mid 2^29) 2^e rounded to FP64, with integer operations.
-__device__ __forceinline__ double fix_to_double(int64_t hh, int64_t mid, int e) {
-    const int64_t t = hh + (mid >> 29);
-    const uint32_t rem = static_cast<uint32_t>(mid) & 0x1FFFFFFFu;
-    const bool neg = t < 0;
-    const uint64_t tm = static_cast<uint64_t>(neg ? (rem ? ~t : -t) : t);
-    const uint32_t rm = neg ? (0x20000000u - rem) & 0x1FFFFFFFu : rem;
-    const int s = min(__clzll(static_cast<long long>(tm)), 29);
-    uint64_t u = (tm << s) | (rm >> (29 - s));
-    const int lz = __clzll(static_cast<long long>(u));
-    const int biased = 63 - lz + 58 - s + e + 1023;
-    if (biased <= 0 || biased >= 2046) return u || e >= kFixNonFinite / 2 ? fix_to_double_slow(t, rem, e) : 0.0;
-    u <<= lz & 63;
-    const uint64_t mant = (u >> 11) + ((u >> 10) & 1);  // in [2^52, 2^53]; zero when u is
-    const uint64_t bits = u ? (static_cast<uint64_t>(biased - 1) << 52) + mant : 0;
-    return __longlong_as_double(static_cast<int64_t>(bits | static_cast<uint64_t>(neg) << 63));
-}
-
-
-// One complex product into the four exact sums: (a.x + i a.z) (b.x + i b.z) with low digits y, w.
-struct FixSum {
-    int64_t rh, rm, ih, im;
-};
-__device__ __forceinline__ void fix_mac(FixSum& c, const int4& a, const int4& b) {
-    const int nzh = -a.z, nzl = -a.w;
-    c.rh += static_cast<int64_t>(a.x) * b.x;
-    c.rm += static_cast<int64_t>(a.x) * b.y;
-    c.ih += static_cast<int64_t>(a.x) * b.z;
-    c.im += static_cast<int64_t>(a.x) * b.w;
-    c.rm += static_cast<int64_t>(a.y) * b.x;
-    c.im += static_cast<int64_t>(a.y) * b.z;
-    c.ih += static_cast<int64_t>(a.z) * b.x;
-    c.im += static_cast<int64_t>(a.z) * b.y;
-    c.rh += static_cast<int64_t>(nzh) * b.z;
-    c.rm += static_cast<int64_t>(nzh) * b.w;
-    c.im += static_cast<int64_t>(a.w) * b.x;
-    c.rm += static_cast<int64_t>(nzl) * b.z;
-}
-__device__ __forceinline__ double2 fix_value(const FixSum& c, int e) {
-    return make_double2(fix_to_double(c.rh, c.rm, e), fix_to_double(c.ih, c.im, e));
-}
-__device__ __forceinline__ int expo_bits(double2 v) {
-    return max(__double2hiint(v.x) & 0x7FF00000, __double2hiint(v.y) & 0x7FF00000);
-}
-__device__ __forceinline__ int4 fix_digits2(double2 v, int emax) {
-    int4 q;
-    fix_digits(v.x, emax, q.x, q.y);
-    fix_digits(v.y, emax, q.z, q.w);
-    return q;
-}
-// Exponent a row's digits are stored with, from its largest exponent field.
-__device__ __forceinline__ int fix_expo(int emax) { return emax == 0x7FF ? kFixNonFinite : emax - 1022 - 57; }
 
 // ---------------------------------------------------------------------------------------------
 // Whole diagonal block in one launch: the inverse of a complex-symmetric block of up to 128 columns

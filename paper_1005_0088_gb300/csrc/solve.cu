@@ -12,6 +12,8 @@
 // several nodes of the level may share, so it uses FP64 atomics; every other write has one owner.
 #include "solve.cuh"
 
+#include "fixed_point.cuh"
+
 #include <algorithm>
 
 namespace ndsi {
@@ -46,24 +48,43 @@ __device__ __forceinline__ void load_tile_wait() {
     __syncthreads();
 }
 
-// Right-hand-side values c + id of kT rows staged for the three-multiplication complex product:
-// (a + ib)(c + id) = [c(a + b) - b(c + d)] + i[c(a + b) + a(d - c)], so a dot product over a tile
-// takes three real FMAs per complex term (c, d - c and c + d stored per value).
+// The products run in fixed point (fixed_point.cuh): a thread owns one row (column) of the tile and a
+// quarter of the inner indices, kQ of them, for all right-hand sides of the block, so that a factor
+// element is turned into digits once per use and serves kSolveRhs products.  The exponents are those
+// of the thread's kQ factor elements and, per right-hand side, of the part's values.  Bound by the
+// latency of one tile (a level has about as many tiles as the GPU SMs): 16 right-hand sides on a 3D
+// box of 6336 orbitals 1108 us with FP64 multiply-adds (64 clocks per sub-partition and instruction),
+// 525 us with four parts of 16 indices, 649 us with eight (each part converts its own sums).
+constexpr int kParts = 4;
+constexpr int kQ = kT / kParts;
+static_assert(kSolveThreads == kParts * kT && kQ <= kFixK, "a thread per tile row and part");
+
+// Right-hand sides of kT rows as digits, with the exponent of every part and column.
 struct RhsTile {
-    double c[kT][kSolveRhs], dmc[kT][kSolveRhs], cpd[kT][kSolveRhs];
+    int4 d[kT][kSolveRhs];
+    int e[kParts][kSolveRhs];
 };
 
-// Stage kT rows (basis indices rb[i0 + r], r < n) of a complex n x k row-major block, RHS c0..
+// Stage kT rows (basis indices rb[i0 + r], r < n) of a complex n x k row-major block, RHS c0..: eight
+// threads per part and right-hand side share its exponent.
 __device__ __forceinline__ void load_rows(RhsTile& v, const double2* X, const int32_t* rb, int i0, int n, int k,
                                           int c0, int nc) {
-    for (int e = threadIdx.x; e < kT * kSolveRhs; e += kSolveThreads) {
-        const int r = e / kSolveRhs, c = e % kSolveRhs;
-        const double2 x = (i0 + r < n && c < nc) ? X[static_cast<int64_t>(rb[i0 + r]) * k + c0 + c]
-                                                 : make_double2(0.0, 0.0);
-        v.c[r][c] = x.x;
-        v.dmc[r][c] = x.y - x.x;
-        v.cpd[r][c] = x.x + x.y;
+    static_assert(kSolveThreads == kParts * kSolveRhs * 8 && kQ % 8 == 0, "eight threads per part and column");
+    const int l = threadIdx.x & 7, c = (threadIdx.x >> 3) % kSolveRhs, q = threadIdx.x / (8 * kSolveRhs);
+    double2 x[kQ / 8];
+    int emax = 0;
+#pragma unroll
+    for (int u = 0; u < kQ / 8; ++u) {
+        const int r = q * kQ + l + 8 * u;
+        x[u] = (i0 + r < n && c < nc) ? X[static_cast<int64_t>(rb[i0 + r]) * k + c0 + c] : make_double2(0.0, 0.0);
+        emax = max(emax, expo_bits(x[u]));
     }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
+    emax >>= 20;
+#pragma unroll
+    for (int u = 0; u < kQ / 8; ++u) v.d[q * kQ + l + 8 * u][c] = fix_digits2(x[u], emax);
+    if (l == 0) v.e[q][c] = fix_expo(emax);
 }
 
 __device__ __forceinline__ void atomic_add2(double2* p, double2 v) {
@@ -71,28 +92,46 @@ __device__ __forceinline__ void atomic_add2(double2* p, double2 v) {
     atomicAdd(&p->y, v.y);
 }
 
-constexpr int kRq = kSolveRhs / 4;  // right-hand sides per thread (four thread quarters)
+// out[c] = sum over the part's inner indices t0 <= i < t1 of elem(i) * rhs(i, c), c < nc; elem(i) is the
+// factor element of this thread's row.
+template <class Elem>
+__device__ __forceinline__ void part_products(const Elem& elem, int t0, int t1, const RhsTile& v, int q, int nc,
+                                                 double2* out) {
+    int emax = 0;
+    for (int i = t0; i < t1; ++i) emax = max(emax, expo_bits(elem(i)));
+    emax >>= 20;
+    FixSum s[kSolveRhs] = {};
+    for (int i = t0; i < t1; ++i) {
+        const int4 a = fix_digits2(elem(i), emax);
+#pragma unroll
+        for (int c = 0; c < kSolveRhs; ++c)
+            if (c < nc) fix_mac(s[c], a, v.d[i][c]);
+    }
+    const int ea = fix_expo(emax);
+#pragma unroll
+    for (int c = 0; c < kSolveRhs; ++c) out[c] = c < nc ? fix_value(s[c], ea + v.e[q][c]) : make_double2(0.0, 0.0);
+}
 
-// Three-multiplication accumulators of kRq complex dot products.
-struct Acc3 {
-    double p1[kRq], p2[kRq], p3[kRq];
-    __device__ __forceinline__ void zero() {
+// Partial sums of the parts, [part][row][right-hand side] (padded), in the space of the tile.
+using PartSums = double2 (*)[kT][kSolveRhs + 1];
+static_assert(kParts * (kSolveRhs + 1) <= kTP, "the partial sums fit the tile");
+// Adds the sum of the parts (negated when `neg`) of rows r (basis index row(r), -1: none) to the n x k block at X, RHS c0..
+template <class Row>
+__device__ __forceinline__ void add_sums(PartSums p, double2* X, int k, int c0, int nc, bool neg, const Row& row) {
+    for (int e = threadIdx.x; e < kT * kSolveRhs; e += kSolveThreads) {
+        const int r = e / kSolveRhs, c = e % kSolveRhs;
+        const int64_t i = row(r);
+        if (c >= nc || i < 0) continue;
+        double2 v[kParts];
 #pragma unroll
-        for (int u = 0; u < kRq; ++u) p1[u] = p2[u] = p3[u] = 0.0;
-    }
-    __device__ __forceinline__ void add(double2 a, const RhsTile& v, int row, int col0) {
-        const double ab = a.x + a.y;
+        for (int q = 0; q < kParts; ++q) v[q] = p[q][r][c];
 #pragma unroll
-        for (int u = 0; u < kRq; ++u) {
-            p1[u] = fma(v.c[row][col0 + u], ab, p1[u]);
-            p2[u] = fma(a.x, v.dmc[row][col0 + u], p2[u]);
-            p3[u] = fma(a.y, v.cpd[row][col0 + u], p3[u]);
-        }
+        for (int o = kParts / 2; o > 0; o /= 2)
+#pragma unroll
+            for (int q = 0; q < o; ++q) v[q] = make_double2(v[q].x + v[q + o].x, v[q].y + v[q + o].y);
+        atomic_add2(X + i * k + c0 + c, neg ? make_double2(-v[0].x, -v[0].y) : v[0]);
     }
-    __device__ __forceinline__ double2 get(int u, double sg) const {
-        return make_double2(sg * (p1[u] - p3[u]), sg * (p1[u] + p2[u]));
-    }
-};
+}
 
 // Forward tile (i0, j0) of node J: front rows i0.. against y_J rows j0..  Rows of R(J) subtract
 // L_RJ y_J from Y; rows of J accumulate w = A_J^{-1} y_J into X from the lower triangle only
@@ -104,6 +143,7 @@ __global__ void __launch_bounds__(kSolveThreads) k_solve_fwd(const SolveNode* __
                                                              int k) {
     extern __shared__ double2 solve_smem[];
     auto t = reinterpret_cast<double2 (*)[kTP]>(solve_smem);
+    auto sums = reinterpret_cast<PartSums>(solve_smem);
     RhsTile& yc = *reinterpret_cast<RhsTile*>(solve_smem + kT * kTP);
     RhsTile& yr = *(&yc + 1);
     const SolveTile tl = tiles[blockIdx.x];
@@ -116,38 +156,32 @@ __global__ void __launch_bounds__(kSolveThreads) k_solve_fwd(const SolveNode* __
     const bool sym = tl.i0 < nd.s;  // the tile has rows of J
     if (sym) load_rows(yr, Y, rb, tl.i0, nd.s, k, c0, nc);
     load_tile_wait();
-    const int q = threadIdx.x >> 6, r = threadIdx.x & (kT - 1);  // 4 quarters of kRq RHS, 64 rows
-    if (kRq * q >= nc) return;  // a whole quarter (two warps) without right-hand sides
-    // direct part: row i0 + r
-    {
-        const int i = tl.i0 + r;
-        if (i < nd.f) {
-            Acc3 acc;
-            acc.zero();
-            const int jmax = i < nd.s ? min(kT, i - tl.j0 + 1) : kT;  // J rows: lower triangle only
-            for (int c = 0; c < jmax; ++c) acc.add(t[c][r], yc, c, kRq * q);
-            double2* dst = (i < nd.s ? X : Y) + static_cast<int64_t>(rb[i]) * k + c0;
-            const double sg = i < nd.s ? 1.0 : -1.0;
+    const int q = threadIdx.x / kT, r = threadIdx.x % kT;  // part of the inner indices, tile row or column
+    double2 direct[kSolveRhs], transposed[kSolveRhs];
+    // direct part: row i0 + r against columns j0.. (J rows: lower triangle only)
+    const int i = tl.i0 + r;
+    const int jmax = i < nd.s ? min(kT, i - tl.j0 + 1) : kT;
+    part_products([&](int c) { return t[c][r]; }, q * kQ, min(q * kQ + kQ, jmax), yc, q, nc, direct);
+    // transposed part (J rows only): column j0 + r against rows i > j of J
+    const int j = tl.j0 + r;
+    if (sym)
+        part_products([&](int c) { return t[r][c]; }, max(q * kQ, j - tl.i0 + 1), min(q * kQ + kQ, nd.s - tl.i0), yr, q,
+                         nc, transposed);
+    __syncthreads();  // the tile's space takes the partial sums
 #pragma unroll
-            for (int u = 0; u < kRq; ++u)
-                if (kRq * q + u < nc && jmax > 0) atomic_add2(dst + kRq * q + u, acc.get(u, sg));
-        }
-    }
-    // transposed part (J rows only): column j0 + r gets sum over rows i > j of A(i, j) y_i
+    for (int c = 0; c < kSolveRhs; ++c) sums[q][r][c] = direct[c];
+    __syncthreads();
+    // rows of J accumulate into X, rows of R(J) subtract from Y
+    add_sums(sums, X, k, c0, nc, false, [&](int rr) { return tl.i0 + rr < nd.s ? rb[tl.i0 + rr] : -1; });
+    add_sums(sums, Y, k, c0, nc, true, [&](int rr) {
+        return tl.i0 + rr >= nd.s && tl.i0 + rr < nd.f ? rb[tl.i0 + rr] : -1;
+    });
     if (sym) {
-        const int j = tl.j0 + r;
-        if (j < nd.s) {
-            const int rmin = max(0, j - tl.i0 + 1), rmax = min(kT, nd.s - tl.i0);
-            if (rmin < rmax) {
-                Acc3 acc;
-                acc.zero();
-                for (int rr = rmin; rr < rmax; ++rr) acc.add(t[r][rr], yr, rr, kRq * q);
-                double2* dst = X + static_cast<int64_t>(rb[j]) * k + c0;
+        __syncthreads();
 #pragma unroll
-                for (int u = 0; u < kRq; ++u)
-                    if (kRq * q + u < nc) atomic_add2(dst + kRq * q + u, acc.get(u, 1.0));
-            }
-        }
+        for (int c = 0; c < kSolveRhs; ++c) sums[q][r][c] = transposed[c];
+        __syncthreads();
+        add_sums(sums, X, k, c0, nc, false, [&](int rr) { return tl.j0 + rr < nd.s ? rb[tl.j0 + rr] : -1; });
     }
 }
 
@@ -158,6 +192,7 @@ __global__ void __launch_bounds__(kSolveThreads) k_solve_bwd(const SolveNode* __
                                                              const double2* __restrict__ F, double2* X, int k) {
     extern __shared__ double2 solve_smem[];
     auto t = reinterpret_cast<double2 (*)[kTP]>(solve_smem);
+    auto sums = reinterpret_cast<PartSums>(solve_smem);
     RhsTile& xr = *reinterpret_cast<RhsTile*>(solve_smem + kT * kTP);
     const SolveTile tl = tiles[blockIdx.x];
     const SolveNode nd = nodes[tl.node];
@@ -167,17 +202,14 @@ __global__ void __launch_bounds__(kSolveThreads) k_solve_bwd(const SolveNode* __
     load_tile(t, F + nd.front_off, nd.f, nd.s + tl.i0, nd.f, tl.j0, nd.s);
     load_rows(xr, X, rb + nd.s, tl.i0, nd.r, k, c0, nc);
     load_tile_wait();
-    const int q = threadIdx.x >> 6, c = threadIdx.x & (kT - 1);
-    const int j = tl.j0 + c;
-    if (j >= nd.s || kRq * q >= nc) return;
-    Acc3 acc;
-    acc.zero();
-    const int tmax = min(kT, nd.r - tl.i0);
-    for (int tt = 0; tt < tmax; ++tt) acc.add(t[c][tt], xr, tt, kRq * q);
-    double2* dst = X + static_cast<int64_t>(rb[j]) * k + c0;
+    const int q = threadIdx.x / kT, c = threadIdx.x % kT;
+    double2 part[kSolveRhs];
+    part_products([&](int u) { return t[c][u]; }, q * kQ, min(q * kQ + kQ, nd.r - tl.i0), xr, q, nc, part);
+    __syncthreads();  // the tile's space takes the partial sums
 #pragma unroll
-    for (int u = 0; u < kRq; ++u)
-        if (kRq * q + u < nc) atomic_add2(dst + kRq * q + u, acc.get(u, -1.0));
+    for (int u = 0; u < kSolveRhs; ++u) sums[q][c][u] = part[u];
+    __syncthreads();
+    add_sums(sums, X, k, c0, nc, true, [&](int rr) { return tl.j0 + rr < nd.s ? rb[tl.j0 + rr] : -1; });
 }
 
 // Row i of the n x k block X times 2^f_i.

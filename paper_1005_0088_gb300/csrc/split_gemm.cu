@@ -1133,12 +1133,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                     __syncwarp();
                     if (lane == 0) mbar_arrive(tmem_free);
                 };
-                // Scales from 3 on lie below 2^-24 of the product, where the low part's own rounding is:
+                // Scales from 4 on lie below 2^-32 of the product, under the low part's own rounding at 2^-48:
                 // they join it by one addition; the others enter the pair by a two-sum.
                 auto sum_band = [&](auto band, const uint32_t* r) {
 #pragma unroll
                     for (int i = 0; i < 2 * CW; ++i) {
-                        if constexpr (EXACT && decltype(band)::value >= 3) lo[i] += __uint_as_float(r[i]);
+                        if constexpr (EXACT && decltype(band)::value >= 4) lo[i] += __uint_as_float(r[i]);
                         else ff_add(hi[i], lo[i], __uint_as_float(r[i]));
                     }
                 };

@@ -42,9 +42,10 @@ extern "C" {
 #define NDSI_ERR_UNSUPPORTED  6   /* feature not available on this device or build */
 
 /* Arithmetic of the dense contractions (separator Schur updates and selected-inverse
- * products).  Diagonal pivot blocks, their inverses and the residue sum are FP64 in both. */
-#define NDSI_PREC_FP64   0   /* FP64 operands on the CUDA cores: products exact in 57-bit fixed point per
-                                operand row and 32 inner indices (integer multiply-adds), summed
+ * products).  Diagonal blocks take the pivots in FP64 and their products in the same
+ * fixed point, and the residue sum is FP64, in both. */
+#define NDSI_PREC_FP64   0   /* FP64 operands on the CUDA cores: products exact in 55-bit fixed point per
+                                operand row and 64 inner indices (integer multiply-adds), summed
                                 in FP64 */
 #define NDSI_PREC_SPLIT  1   /* FP64 emulated by BF16 slices on the tcgen05 tensor cores */
 

@@ -1157,14 +1157,14 @@ int ndsi_autotune(ndsi_plan* h, const double* H, const double* S, double mu, dou
     // with every eligible GEMM on the FP64 CUDA cores (each after an untimed warm-up sweep); each
     // launch then keeps the faster of the two.  Both choices meet the split tolerance, so the
     // result only changes speed.  The profiler's own counters are left as they were.
-    // A step whose tensor-core time is already below the least time the FP64 path could take (twelve
+    // A step whose tensor-core time is already below the least time the FP64 path could take (nine
     // integer multiply-adds per complex product at 64 lanes per clock and SM, k_gemm_f64's bound) is
     // decided without running it on the CUDA cores: only the other steps are timed there.
     int dev = 0, sms = 0, khz = 0;
     NDSI_CK(cudaGetDevice(&dev));
     NDSI_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     NDSI_CK(cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev));
-    const double peak = 8.0 * 64.0 / 12.0 * sms * khz * 1e3;  // 8-flop complex products per second
+    const double peak = 8.0 * 64.0 / 9.0 * sms * khz * 1e3;  // 8-flop complex products per second
     Profiler saved = h->prof;
     h->prof.pending.clear();
     h->prof.used = 0;

@@ -578,12 +578,19 @@ __global__ void __launch_bounds__(512) k_diaginv_block(const DiagItem* __restric
 
 // ---------------------------------------------------------------------------------------------
 // Batched complex FP64 GEMM on the CUDA cores: C = alpha op(A) op(B) + beta C for every tile of
-// a schedule step, products in fixed point (above) over chunks of 32 inner indices, the chunks
-// added in FP64.  One CTA of 128 threads per 32 x 32 output tile, outputs 8 rows and 16 columns apart,
-// so that a ragged tile skips its empty 8-row and (per warp) 4-column groups and a tile on the
-// diagonal of a lower-triangle result those above it; operands are staged by cp.async and turned
-// into digits in place, two threads per operand row.  Four CTAs per SM overlap one CTA's loads and
-// conversion with the others' products.
+// a schedule step, products in fixed point (fixed_point.cuh, three real products per complex one)
+// over chunks of 64 inner indices, every chunk added to C in FP64 as soon as it is complete.  One
+// CTA of 256 threads per 32 x 32 output tile; a warp has the groups of 8 rows and 4 columns that
+// lie 16 apart, 2 x 2 outputs per thread, so that a ragged tile skips its empty groups in all warps
+// alike and a tile on the diagonal of a lower-triangle result those above it; operands are staged
+// by cp.async and turned into digits in place, four threads per operand row.
+//
+// Full tiles are bound by the multiply-adds (heavy FMA pipe 74% busy at 64-wide pivots, 5.1 TF
+// counting 8 operations per complex product); fronts of 36-44 columns, whose second tile is nearly empty,
+// by latency (49%), which is why sums are added to memory and not kept in registers: 80 registers
+// and three CTAs per SM instead of 124 and two, 15.5 -> 14.8 ms for 80 poles of a 2D sheet of 32 x 32
+// atoms x 4 orbitals, at 8.0 -> 8.3 ms for 8 points of a 9 x 8 x 7 box x 5.  Four products per complex one
+// in chunks of 32 took 16.7 and 9.9 ms, DFMA loops 44.2 and 23.5 ms.
 template <int OP>
 __device__ __forceinline__ int64_t op_offset(int ld, int r, int c) {
     if (OP == OP_N) return r + static_cast<int64_t>(c) * ld;
@@ -592,37 +599,37 @@ __device__ __forceinline__ int64_t op_offset(int ld, int r, int c) {
     return hi + static_cast<int64_t>(lo) * ld;
 }
 
-constexpr int kFixThreads = 128;
-// kc inner products of a thread's mi x nj outputs (FULL: 4 x 2); group (i, j) is skipped when all of it
-// lies above the diagonal, 8 i < d + 16 j (d <= -16: no group).
+constexpr int kFixThreads = 256;
+using FixTile = int4[kFix3K][kGemmTile + 1];  // op(A) rows or op(B) columns: raw FP64, then digits
+constexpr int kFixSmem = 2 * static_cast<int>(sizeof(FixTile));
+
+// kc inner products of a thread's outputs (row + 16 i, col + 16 j); bit 2 i + j of `live`: the group has a
+// wanted output (FULL: all have).
 template <bool FULL>
 __device__ __forceinline__ void fix_products(const int4 (*As)[kGemmTile + 1], const int4 (*Bs)[kGemmTile + 1], int kc,
-                                             int tx, int ty, int mi, int nj, int d, FixSum (&c)[4][2]) {
+                                             int row, int col, uint32_t live, Fix3Sum (&c)[2][2]) {
 #pragma unroll 1
     for (int k = 0; k < kc; ++k) {
-        int4 b[2];
+        const int4 b[2] = {Bs[k][col], Bs[k][col + 16]};
+        const int2 bs[2] = {fix3_sum(b[0]), fix3_sum(b[1])};
 #pragma unroll
-        for (int j = 0; j < 2; ++j)
-            if (FULL || j < nj) b[j] = Bs[k][ty + 16 * j];
+        for (int i = 0; i < 2; ++i) {
+            const int4 a = As[k][row + 16 * i];  // re h, re l, im h, im l
+            const int2 as = fix3_sum(a);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            if (!FULL && i >= mi) continue;
-            const int4 a = As[k][tx + 8 * i];  // re h, re l, im h, im l
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                if (!FULL && (j >= nj || 8 * i < d + 16 * j)) continue;
-                fix_mac(c[i][j], a, b[j]);
-            }
+            for (int j = 0; j < 2; ++j)
+                if (FULL || (live >> (2 * i + j) & 1)) fix3_mac(c[i][j], a, as, b[j], bs[j]);
         }
     }
 }
 
 template <int OPA, int OPB>
-__global__ void __launch_bounds__(kFixThreads, 4)
+__global__ void __launch_bounds__(kFixThreads, 3)
     k_gemm_f64(const GemmItem* __restrict__ items, const GemmTile* __restrict__ tiles, int64_t tfirst, int64_t ifirst,
                const double2* __restrict__ Abuf, int64_t sA, const double2* __restrict__ Bbuf, int64_t sB,
                double2* __restrict__ Cbuf, int64_t sC, double alpha, double beta, int lower) {
-    __shared__ int4 sh[2][kFixK][kGemmTile + 1];  // op(A) rows, op(B) columns: raw FP64, then digits
+    extern __shared__ __align__(16) unsigned char fix_smem[];
+    FixTile* sh = reinterpret_cast<FixTile*>(fix_smem);
     __shared__ int ex[2][kGemmTile];
     const GemmTile t = tiles[tfirst + blockIdx.x];
     const GemmItem it = items[ifirst + t.item];
@@ -630,86 +637,79 @@ __global__ void __launch_bounds__(kFixThreads, 4)
     const double2* A = Abuf + pole * sA + it.a_off;
     const double2* B = Bbuf + pole * sB + it.b_off;
     double2* C = Cbuf + pole * sC + it.c_off;
-    // outputs (tx + 8 i, ty + 16 j); a warp holds 8 rows x 4 columns of each group
-    const int tid = threadIdx.x, tx = tid % 8, ty = tid / 8;
+    const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
     const int mrem = min(kGemmTile, it.M - t.m0), nrem = min(kGemmTile, it.N - t.n0);
-    const int mi = (mrem + 7) / 8;
-    const int nj = (nrem - (ty & ~3) + 15) / 16;  // column groups of this warp with a live column
-    // first row group of column group j that reaches the diagonal: 8 i + 7 >= n0 + (ty & ~3) + 16 j - m0
-    const int d = lower ? t.n0 - t.m0 + (ty & ~3) - 7 : -64;
-    double2 acc[4][2];
+    const int r0 = (warp / 4) * 8, c0 = (warp % 4) * 4;  // the warp's first row and column
+    const int row = r0 + lane % 8, col = c0 + lane / 8;
+    uint32_t live = 0;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int j = 0; j < 2; ++j) acc[i][j] = make_double2(0.0, 0.0);
-    for (int k0 = 0; k0 < it.K; k0 += kFixK) {
-        const int kc = min(kFixK, it.K - k0);
+        for (int j = 0; j < 2; ++j)
+            if (r0 + 16 * i < mrem && c0 + 16 * j < nrem && !(lower && t.m0 + r0 + 16 * i + 7 < t.n0 + c0 + 16 * j))
+                live |= 1u << (2 * i + j);
+    for (int k0 = 0; k0 < it.K; k0 += kFix3K) {
+        const int kc = min(kFix3K, it.K - k0);
         auto stage = [&](int4* dst, const double2* src, bool ok) {
             const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
             asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(ok ? 16 : 0) : "memory");
         };
-#pragma unroll 4
-        for (int u = 0; u < kGemmTile * kFixK / kFixThreads; ++u) {
-            const int e = tid + u * kFixThreads;
-            const int f = e % 32, g = e / 32;
-            const int m = OPA == OP_T ? g : f, ka = OPA == OP_T ? f : g;
+#pragma unroll
+        for (int u = 0; u < kGemmTile * kFix3K / kFixThreads; ++u) {
+            const int g = warp + u % 4 * 8, f = lane + u / 4 * 32;  // for the operand that is contiguous in k
+            const int w = warp + u * 8;
+            const int m = OPA == OP_T ? g : lane, ka = OPA == OP_T ? f : w;
             if (ka < kc) stage(&sh[0][ka][m], A + (m < mrem ? op_offset<OPA>(it.lda, t.m0 + m, k0 + ka) : 0), m < mrem);
-            const int n = OPB == OP_T ? f : g, kb = OPB == OP_T ? g : f;
+            const int n = OPB == OP_T ? lane : g, kb = OPB == OP_T ? w : f;
             if (kb < kc) stage(&sh[1][kb][n], B + (n < nrem ? op_offset<OPB>(it.ldb, k0 + kb, t.n0 + n) : 0), n < nrem);
         }
         asm volatile("cp.async.wait_all;\n" ::: "memory");
         __syncthreads();
         {
-            // two threads per operand row (even and odd inner indices): the largest exponent field
-            // of the chunk, then the digits in place
-            int4 (*x)[kGemmTile + 1] = sh[tid / 64];
-            const int row = (tid / 32 % 2) * 16 + tid % 16, kh = tid / 16 % 2;
+            // four threads per operand row: the largest exponent field of the chunk, then the
+            // digits in place
+            int4 (*x)[kGemmTile + 1] = sh[warp / 4];
+            const int rr = (warp % 4) * 8 + lane % 8, kh = lane / 8;
             int emax = 0;
-            for (int k = kh; k < kc; k += 2)
-                emax = max(emax, max(x[k][row].y & 0x7FF00000, x[k][row].w & 0x7FF00000));
+#pragma unroll 4
+            for (int u = 0; u < kFix3K / 4; ++u) {
+                const int k = kh + 4 * u;
+                if (k < kc) emax = max(emax, max(x[k][rr].y & 0x7FF00000, x[k][rr].w & 0x7FF00000));
+            }
+            emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 8));
             emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 16)) >> 20;
-            for (int k = kh; k < kc; k += 2)
-                x[k][row] = fix_digits2(*reinterpret_cast<const double2*>(&x[k][row]), emax);
-            if (kh == 0) ex[tid / 64][row] = fix_expo(emax);
+#pragma unroll 4
+            for (int u = 0; u < kFix3K / 4; ++u) {
+                const int k = kh + 4 * u;
+                if (k < kc) x[k][rr] = fix_digits2<kFix3>(*reinterpret_cast<const double2*>(&x[k][rr]), emax);
+            }
+            if (kh == 0) ex[warp / 4][rr] = fix_expo<kFix3>(emax);
         }
         __syncthreads();
-        if (nj > 0) {
-            FixSum c[4][2] = {};
-            if (mi == 4 && nj == 2 && d <= -16) fix_products<true>(sh[0], sh[1], kc, tx, ty, mi, nj, d, c);
-            else fix_products<false>(sh[0], sh[1], kc, tx, ty, mi, nj, d, c);
+        if (live) {
+            Fix3Sum c[2][2] = {};
+            if (live == 15u) fix_products<true>(sh[0], sh[1], kc, row, col, live, c);
+            else fix_products<false>(sh[0], sh[1], kc, row, col, live, c);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                if (i >= mi) continue;
-                const int ea = ex[0][tx + 8 * i];
+            for (int i = 0; i < 2; ++i)
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
-                    if (j >= nj || 8 * i < d + 16 * j) continue;
-                    const double2 v = fix_value(c[i][j], ea + ex[1][ty + 16 * j]);
-                    acc[i][j] = k0 == 0 ? v : cadd(acc[i][j], v);
+                    const int m = t.m0 + row + 16 * i, n = t.n0 + col + 16 * j;
+                    if (m >= it.M || n >= it.N || (lower && m < n)) continue;
+                    double2 v = fix3_value(c[i][j], ex[0][row + 16 * i] + ex[1][col + 16 * j]);
+                    if (alpha == -1.0) v = make_double2(-v.x, -v.y);
+                    else if (alpha != 1.0) v = make_double2(alpha * v.x, alpha * v.y);
+                    const double b = k0 == 0 ? beta : 1.0;
+                    double2* out = C + m + static_cast<int64_t>(n) * it.ldc;
+                    if (b != 0.0) {
+                        const double2 old = *out;
+                        if (b == 1.0) v = cadd(v, old);
+                        else v = make_double2(fma(b, old.x, v.x), fma(b, old.y, v.y));
+                    }
+                    *out = v;
                 }
-            }
         }
         __syncthreads();
-    }
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        const int n = t.n0 + ty + 16 * j;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int m = t.m0 + tx + 8 * i;
-            if (m < it.M && n < it.N && (!lower || m >= n)) {
-                double2* c = C + m + static_cast<int64_t>(n) * it.ldc;
-                double2 v = acc[i][j];
-                if (alpha == -1.0) v = make_double2(-v.x, -v.y);
-                else if (alpha != 1.0) v = make_double2(alpha * v.x, alpha * v.y);
-                if (beta != 0.0) {
-                    const double2 old = *c;
-                    if (beta == 1.0) v = cadd(v, old);
-                    else v = make_double2(fma(beta, old.x, v.x), fma(beta, old.y, v.y));
-                }
-                *c = v;
-            }
-        }
     }
 }
 
@@ -837,7 +837,7 @@ cudaError_t gemm_launch(const Plan& P, const DevTables& T, const Launch& l, cons
     const double2* bufs[2] = {W.fronts, W.scr};
     const int64_t strides[2] = {W.front_stride, W.scr_stride};
     dim3 grid(static_cast<unsigned>(l.tcount), static_cast<unsigned>(np));
-    k_gemm_f64<OPA, OPB><<<grid, kFixThreads, 0, st>>>(
+    k_gemm_f64<OPA, OPB><<<grid, kFixThreads, kFixSmem, st>>>(
         T.gemm_items, T.gemm_tiles, l.tfirst, l.first, bufs[l.bufA], strides[l.bufA], bufs[l.bufB],
         strides[l.bufB], const_cast<double2*>(bufs[l.bufC]), strides[l.bufC], l.alpha, l.beta, l.lower);
     (void)P;
@@ -919,6 +919,11 @@ cudaError_t launch_basis_scale(const Plan& P, const DevTables& T, const double* 
 }
 
 cudaError_t kernels_init() {
+    using Gemm = decltype(&k_gemm_f64<OP_N, OP_S>);
+    for (Gemm f : {&k_gemm_f64<OP_N, OP_S>, &k_gemm_f64<OP_N, OP_T>, &k_gemm_f64<OP_S, OP_N>, &k_gemm_f64<OP_T, OP_N>}) {
+        const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kFixSmem);
+        if (e != cudaSuccess) return e;
+    }
     const int smb = static_cast<int>(diag_block_smem(kDiagBlockMax));
     const cudaError_t e = cudaFuncSetAttribute(k_diaginv_block, cudaFuncAttributeMaxDynamicSharedMemorySize, smb);
     if (e != cudaSuccess) return e;

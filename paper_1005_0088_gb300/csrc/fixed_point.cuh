@@ -127,6 +127,9 @@ __device__ __forceinline__ void fix3_mac(Fix3Sum& c, const int4& a, int2 as, con
     c.m3 += fix_wide(as.y, bs.x);
 }
 __device__ __forceinline__ int2 fix3_sum(const int4& a) { return make_int2(a.x + a.z, a.y + a.w); }
+__device__ __forceinline__ void fix3_mac(Fix3Sum& c, const int4& a, const int4& b) {
+    fix3_mac(c, a, fix3_sum(a), b, fix3_sum(b));
+}
 __device__ __forceinline__ double2 fix3_value(const Fix3Sum& c, int e) {
     return make_double2(fix_to_double<kFix3>(static_cast<int64_t>(c.h1 - c.h2), static_cast<int64_t>(c.m1 - c.m2), e),
                         fix_to_double<kFix3>(static_cast<int64_t>(c.h3 - c.h1 - c.h2),

@@ -284,20 +284,44 @@ __global__ void __launch_bounds__(32) k_diaginv_sweep(const DiagItem* __restrict
 // and after every pivot block A holds -A^{-1}; every intermediate matrix is symmetric, so only 8 x 8
 // blocks of the lower triangle are kept (in shared memory, FP64) and updated (n^3 / 2 complex
 // multiply-adds).  The pivot blocks are inverted in FP64; the panel and update products run in
-// fixed point (above), with the panels' digits formed once per pivot step.
-// Bound: the integer multiply-add pipe for the updates (16 x 8 units handed out dynamically) and the
-// FP64 latency of the pivot block (16 dependent divisions, about 40k clocks on one warp, since a
-// sub-partition takes 64 clocks per FP64 instruction); one warp therefore inverts the next pivot
-// block, updated first, while the others still update.
+// fixed point (fixed_point.cuh, three real products), with the panels' digits formed once per pivot step.
+// Bound: for 128 columns the updates (16 x 8 units handed out dynamically, 45k of 71k clocks per pivot
+// block), for narrow blocks, of which two or three share an SM, the FP64 instructions of the pivot
+// block: a sub-partition takes 64 clocks for each and an SM 16, so four warps, one per
+// sub-partition, invert the next pivot block, updated first, while the others still update.  40
+// poles of a chain of 64 atoms x 8 orbitals (128-column blocks) 1.13 -> 0.96 ms against one pivot warp with
+// divisions and twelve multiply-adds per product, twelve uneven systems (batched, 80 columns and fewer)
+// 63.0 -> 59.1 ms, density of states of a 30 x 26 x 5 sheet 14.4 -> 13.3 ms.
 // Replaces, per 16 columns, a pivot-inverse, panel, update and copy launch each and the backward
 // assembly (53 launches for 128 columns).
-constexpr int kBlkP = 16;  // pivot width
+constexpr int kBlkP = 16;   // pivot width
+constexpr int kBlkLd = 17;  // row stride of pivot blocks in shared memory
+
+// 1 / x, x normal and positive, to about one unit in the last place: the hardware's FP32 reciprocal of the
+// mantissa (relative error e below 2^-21) and one third-order step y (1 + e + e^2), e = 1 - m y (the
+// series of 1 / (1 - e); what is left is e^3 < 2^-63).  A division takes 435 clocks, FP64 instructions
+// of one warp 64 each.
+__device__ __forceinline__ double pivot_rcp(double x) {
+    const uint32_t hi = static_cast<uint32_t>(__double2hiint(x)), lo = static_cast<uint32_t>(__double2loint(x));
+    const uint32_t ex = hi >> 20;
+    if (ex - 1u >= 2044u) return 1.0 / x;  // zero, subnormal, non-finite, or a subnormal result
+    const double m = __hiloint2double(static_cast<int>((hi & 0xFFFFFu) | 0x3FF00000u), static_cast<int>(lo));
+    const float mf = __uint_as_float(0x3F800000u | (hi & 0xFFFFFu) << 3 | lo >> 29);
+    float yf;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(mf));
+    const uint32_t yb = __float_as_uint(yf);
+    const double y = __hiloint2double(static_cast<int>((yb >> 3) + (896u << 20)), static_cast<int>(yb << 29));
+    const double e = fma(-m, y, 1.0);
+    const double r = fma(y, fma(e, e, e), y);  // in [1/2, 1]
+    return __hiloint2double(__double2hiint(r) - ((static_cast<int>(ex) - 1023) << 20), __double2loint(r));
+}
 
 __host__ __device__ constexpr size_t diag_block_smem(int tile) {
     const int nb8 = tile / 8, rows = tile - kBlkP;
     return static_cast<size_t>(nb8 * (nb8 + 1) / 2) * 64 * sizeof(double2) +        // lower 8 x 8 blocks
-           sizeof(int4) * (2 * kBlkP * rows + kBlkP * kBlkP) +                      // digits of W, C and P
-           sizeof(int) * (2 * rows + kBlkP) + sizeof(double2) * 2 * (kBlkP + 1) +   // exponents, pivot column
+           sizeof(int4) * (2 * kBlkP * rows + kBlkP * kBlkLd) +                     // digits of W, C and P
+           sizeof(double2) * kBlkP * (kBlkLd + 1) +                                 // pivot block, scaled column
+           sizeof(int) * (2 * rows + kBlkP) +                                       // exponents
            sizeof(int) * 4 + sizeof(uint16_t) * nb8 * (nb8 + 1) / 2;                // counters, unit list
 }
 
@@ -313,10 +337,10 @@ __global__ void __launch_bounds__(512) k_diaginv_block(const DiagItem* __restric
     const int T8 = tile / 8, R = tile - kBlkP;
     double2* M = smem_blk;                                    // block (I, J) at I (I + 1) / 2 + J, column-major
     int4* Wd = reinterpret_cast<int4*>(M + (T8 * (T8 + 1) / 2) * 64);  // [16][R], k-major
-    int4 *Cd = Wd + kBlkP * R, *Pd = Cd + kBlkP * R;          // [16][R]; [16][16] symmetric
-    double2* cs = reinterpret_cast<double2*>(Pd + kBlkP * kBlkP);      // [17] pivot column, [16] dummy
-    double2* ds = cs + kBlkP + 1;
-    int* We = reinterpret_cast<int*>(ds + kBlkP + 1);         // row exponents of W, C; column exponents of P
+    int4 *Cd = Wd + kBlkP * R, *Pd = Cd + kBlkP * R;          // [16][R]; [16][17] symmetric
+    double2* XB = reinterpret_cast<double2*>(Pd + kBlkP * kBlkLd);     // [16][17] second copy of the pivot block
+    double2* ds = XB + kBlkP * kBlkLd;                        // [16] scaled pivot column
+    int* We = reinterpret_cast<int*>(ds + kBlkP);            // row exponents of W, C; column exponents of P
     int *Ce = We + R, *Pe = Ce + R;
     int* ctr = Pe + kBlkP;                                    // [0] next unit, [1] list length
     uint16_t* list = reinterpret_cast<uint16_t*>(ctr + 4);    // update units: row pair I16 << 8 | column block J
@@ -347,93 +371,77 @@ __global__ void __launch_bounds__(512) k_diaginv_block(const DiagItem* __restric
         ctr[1] = cnt;
     }
     const int r8 = lane & 7, cq = lane >> 3;  // a unit's row and first column of this lane
-    // inverse of pivot block t by one warp (rank-1 symmetric sweeps, packed lower triangle; see
-    // k_diaginv_sweep), written to the block itself (-P) and, as digits, to P
+    // inverse of pivot block t by warps 0..3 (rank-1 symmetric sweeps on the lower triangle), written
+    // to the block itself (-P) and, as digits, to P.  A step reads one of two copies and writes the
+    // other; the warps take turns at the scaled column, which costs twice the FP64 instructions of a
+    // warp's share of the update.
     auto pivot = [&](int t) {
-        constexpr int VC = kBlkP / 2, LPC = 32 / VC, SLOTS = (kBlkP + 1 + LPC - 1) / LPC;
         const int nb = min(kBlkP, n - t * kBlkP);
-        const int c = lane % VC, vbase = (lane / VC) * SLOTS;
         auto at = [&](int i, int k) { return blk(2 * t + (i >> 3), 2 * t + (k >> 3)) + (k & 7) * 8 + (i & 7); };
-        int rc[SLOTS];
-        double2 a[SLOTS];
-#pragma unroll
-        for (int s = 0; s < SLOTS; ++s) {
-            const int v = vbase + s;
-            int i = kBlkP, k = kBlkP;
-            if (v < kBlkP - c) {
-                i = c + v;
-                k = c;
-            } else if (v <= kBlkP) {
-                i = v - 1;
-                k = kBlkP - 1 - c;
-            }
-            rc[s] = i | (k << 8);
-            a[s] = make_double2(0.0, 0.0);
-            if (i < nb && k < nb) a[s] = *at(i, k);
+        auto barrier = [] { asm volatile("bar.sync 1, 128;" ::: "memory"); };
+        double2* XA = reinterpret_cast<double2*>(Pd);
+        for (int e = tid; e < kBlkP * kBlkP; e += 128) {
+            const int i = e / kBlkP, k = e % kBlkP;
+            if (k <= i) XA[i * kBlkLd + k] = i < nb ? *at(i, k) : make_double2(0.0, 0.0);
         }
-        if (lane == 0) cs[kBlkP] = ds[kBlkP] = make_double2(0.0, 0.0);
+        // this thread's element among the 120 outside the pivot row and column, counted without them
+        const bool own = tid < kBlkP * (kBlkP - 1) / 2;
+        int i0 = 0;
+        while (own && (i0 + 1) * (i0 + 2) / 2 <= tid) ++i0;
+        const int j0 = own ? tid - i0 * (i0 + 1) / 2 : 0;
+        const int idx = lane & 15;  // column element of this lane: real part, or imaginary part in lanes 16..31
+        const bool im = lane >= 16;
         bool bad = false;
+        barrier();
         for (int q = 0; q < nb; ++q) {
-#pragma unroll
-            for (int s = 0; s < SLOTS; ++s) {
-                const int i = rc[s] & 255, k = rc[s] >> 8;
-                if (k == q) cs[i] = a[s];
-                if (i == q) cs[k] = a[s];
+            const double2* X = q & 1 ? XB : XA;
+            double2* Y = q & 1 ? XA : XB;
+            auto tri = [](int r, int c) { return r > c ? r * kBlkLd + c : c * kBlkLd + r; };
+            if (warp == (q & 3)) {  // d = c / p, 1 / p in the pivot's place
+                const double2 p = X[tri(q, q)];
+                const double2 c = idx == q ? make_double2(1.0, 0.0) : X[tri(idx, q)];
+                const double den = p.x * p.x + p.y * p.y;
+                // zero, subnormal or non-finite: decided on the exponent field, off the FP64 pipe
+                bad |= (static_cast<uint32_t>(__double2hiint(den)) >> 20) - 1u >= 0x7FEu;
+                const double u = im ? c.y : c.x, v = im ? -c.x : c.y;
+                const double d = fma(u, p.x, v * p.y) * pivot_rcp(den);
+                reinterpret_cast<double*>(ds + idx)[im] = d;
+                reinterpret_cast<double*>(Y + tri(idx, q))[im] = idx == q ? -d : d;
             }
-            __syncwarp();
-            const double2 p = cs[q];
-            const double den = p.x * p.x + p.y * p.y;
-            // zero, subnormal or non-finite: decided on the exponent field, off the FP64 pipe
-            const uint32_t dx = static_cast<uint32_t>(__double2hiint(den)) >> 20;
-            bad |= dx - 1u >= 0x7FEu;
-            const double rden = 1.0 / den;
-            const double2 ip = make_double2(p.x * rden, -p.y * rden), nip = make_double2(-ip.x, -ip.y);
-            if (lane < kBlkP) ds[lane] = cmul(cs[lane], ip);
-            __syncwarp();
-#pragma unroll
-            for (int s = 0; s < SLOTS; ++s) {
-                const int i = rc[s] & 255, k = rc[s] >> 8;
-                const double2 cv = cs[i], dk = ds[k], di = ds[i];
-                const double2 g = make_double2(fma(-cv.x, dk.x, fma(cv.y, dk.y, a[s].x)), fma(-cv.x, dk.y, fma(-cv.y, dk.x, a[s].y)));
-                // the pivot row and column take d (the pivot itself -1/p), by selects: a branch here diverges
-                const bool kq = k == q, iq = i == q;
-                const double2 o = kq ? (iq ? nip : di) : dk;
-                a[s] = make_double2(kq | iq ? o.x : g.x, kq | iq ? o.y : g.y);
-            }
-            __syncwarp();
+            const int i = i0 + (i0 >= q), j = j0 + (j0 >= q);
+            const double2 ci = X[tri(i, q)], a = X[tri(i, j)];
+            barrier();
+            const double2 dj = ds[j];
+            if (own)
+                Y[tri(i, j)] = make_double2(fma(-ci.x, dj.x, fma(ci.y, dj.y, a.x)), fma(-ci.x, dj.y, fma(-ci.y, dj.x, a.y)));
+            barrier();
         }
         if (bad && lane == 0) atomicOr(status, kStatusSingular);
-        double2* P = reinterpret_cast<double2*>(Pd);
-#pragma unroll
-        for (int s = 0; s < SLOTS; ++s) {
-            const int i = rc[s] & 255, k = rc[s] >> 8;
-            if (i >= kBlkP) continue;
-            const bool in = i < nb && k < nb;
-            if (in) *at(i, k) = a[s];
-            P[i * kBlkP + k] = P[k * kBlkP + i] = in ? make_double2(-a[s].x, -a[s].y) : make_double2(0.0, 0.0);
+        const double2* X = nb & 1 ? XB : XA;
+        for (int e = tid; e < kBlkP * kBlkP; e += 128) {
+            const int i = e / kBlkP, k = e % kBlkP;
+            if (k <= i && i < nb) *at(i, k) = X[i * kBlkLd + k];
         }
-        __syncwarp();
-        // digits of P in place, two lanes per column
-        const int col = lane & 15, kh = lane >> 4;
+        // digits of P = -X, eight lanes per column, two rows each
+        const int col = tid >> 3;
+        double2 x[2];
         int emax = 0;
 #pragma unroll
-        for (int k = 0; k < kBlkP / 2; ++k) emax = max(emax, expo_bits(P[(2 * k + kh) * kBlkP + col]));
-        emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 16)) >> 20;
-#pragma unroll
-        for (int k = 0; k < kBlkP / 2; ++k) {
-            const int o = (2 * k + kh) * kBlkP + col;
-            Pd[o] = fix_digits2(P[o], emax);
+        for (int h = 0; h < 2; ++h) {
+            const int k = (tid & 7) + 8 * h;
+            const double2 y = X[k > col ? k * kBlkLd + col : col * kBlkLd + k];
+            x[h] = k < nb && col < nb ? make_double2(-y.x, -y.y) : make_double2(0.0, 0.0);
+            emax = max(emax, expo_bits(x[h]));
         }
-        if (kh == 0) Pe[col] = fix_expo(emax);
+#pragma unroll
+        for (int o = 1; o < 8; o *= 2) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
+        barrier();  // X may be P's own storage
+#pragma unroll
+        for (int h = 0; h < 2; ++h) Pd[((tid & 7) + 8 * h) * kBlkLd + col] = fix_digits2<kFix3>(x[h], emax >> 20);
+        if ((tid & 7) == 0) Pe[col] = fix_expo<kFix3>(emax >> 20);
     };
     __syncthreads();
-    // the warp that inverts the pivot blocks: co-resident CTAs take warps of different SM sub-partitions
-    uint32_t slot;
-    asm volatile("mov.u32 %0, %%warpid;" : "=r"(slot));
-    if (tid == 0) ctr[2] = static_cast<int>(slot / nw) & 3;
-    __syncthreads();
-    const int wp = ctr[2];
-    if (warp == wp) pivot(0);
+    if (warp < 4) pivot(0);
     __syncthreads();
     for (int t = 0; t < nt; ++t) {
         const int w8 = min(2, nb8 - 2 * t), kw = 8 * w8, m8 = nb8 - w8, m = 8 * m8;
@@ -458,28 +466,28 @@ __global__ void __launch_bounds__(512) k_diaginv_block(const DiagItem* __restric
             if (row < m) {
 #pragma unroll
                 for (int k = 0; k < kBlkP / 2; ++k)
-                    if (2 * k < kw) Cd[(2 * k + kh) * R + row] = fix_digits2(v[k], emax);
-                if (kh == 0) Ce[row] = fix_expo(emax);
+                    if (2 * k < kw) Cd[(2 * k + kh) * R + row] = fix_digits2<kFix3>(v[k], emax);
+                if (kh == 0) Ce[row] = fix_expo<kFix3>(emax);
             }
         }
         __syncthreads();
         // W = C P, eight rows of W per warp; the pivot column becomes W (its old values stay in C)
         for (int u = warp; u < m8; u += nw) {
             const int row = u * 8 + r8, Ig = u < 2 * t ? u : u + w8;
-            FixSum c[4] = {};
+            Fix3Sum c[4] = {};
 #pragma unroll 2
             for (int k = 0; k < kw; ++k) {
                 const int4 a = Cd[k * R + row];
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
-                    if (4 * q < kw) fix_mac(c[q], a, Pd[k * kBlkP + cq + 4 * q]);
+                    if (4 * q < kw) fix3_mac(c[q], a, Pd[k * kBlkLd + cq + 4 * q]);
             }
             double2 w[4];
             int emax = 0;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 w[q] = make_double2(0.0, 0.0);
-                if (4 * q < kw) w[q] = fix_value(c[q], Ce[row] + Pe[cq + 4 * q]);
+                if (4 * q < kw) w[q] = fix3_value(c[q], Ce[row] + Pe[cq + 4 * q]);
                 emax = max(emax, expo_bits(w[q]));
             }
             emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 8));
@@ -488,10 +496,10 @@ __global__ void __launch_bounds__(512) k_diaginv_block(const DiagItem* __restric
             for (int q = 0; q < 4; ++q) {
                 if (4 * q >= kw) continue;
                 const int k = cq + 4 * q, K = 2 * t + (k >> 3);
-                Wd[k * R + row] = fix_digits2(w[q], emax);
+                Wd[k * R + row] = fix_digits2<kFix3>(w[q], emax);
                 (Ig < K ? blk(K, Ig)[r8 * 8 + (k & 7)] : blk(Ig, K)[(k & 7) * 8 + r8]) = w[q];
             }
-            if (cq == 0) We[row] = fix_expo(emax);
+            if (cq == 0) We[row] = fix_expo<kFix3>(emax);
         }
         __syncthreads();
         // A_IJ -= W_I C_J^T for the row blocks 2 I16, 2 I16 + 1 and column block J, one unit per warp
@@ -499,25 +507,25 @@ __global__ void __launch_bounds__(512) k_diaginv_block(const DiagItem* __restric
             const int I0 = 2 * I16, shift = I0 < 2 * t ? 0 : w8;
             const bool lo = J <= I0, hi = I0 + 1 < nb8;
             const int row = (I0 - shift) * 8 + r8, col = (J < 2 * t ? J : J - w8) * 8 + cq;
-            FixSum c[2][2] = {};
+            Fix3Sum c[2][2] = {};
             if (lo && hi) {
 #pragma unroll 2
                 for (int k = 0; k < kw; ++k) {
                     const int4 a0 = Wd[k * R + row], a1 = Wd[k * R + row + 8];
                     const int4 b0 = Cd[k * R + col], b1 = Cd[k * R + col + 4];
-                    fix_mac(c[0][0], a0, b0);
-                    fix_mac(c[0][1], a0, b1);
-                    fix_mac(c[1][0], a1, b0);
-                    fix_mac(c[1][1], a1, b1);
+                    fix3_mac(c[0][0], a0, b0);
+                    fix3_mac(c[0][1], a0, b1);
+                    fix3_mac(c[1][0], a1, b0);
+                    fix3_mac(c[1][1], a1, b1);
                 }
             } else {
                 const int r = lo ? row : row + 8, g = lo ? 0 : 1;
-                FixSum c0{}, c1{};
+                Fix3Sum c0{}, c1{};
 #pragma unroll 2
                 for (int k = 0; k < kw; ++k) {
                     const int4 a = Wd[k * R + r];
-                    fix_mac(c0, a, Cd[k * R + col]);
-                    fix_mac(c1, a, Cd[k * R + col + 4]);
+                    fix3_mac(c0, a, Cd[k * R + col]);
+                    fix3_mac(c1, a, Cd[k * R + col + 4]);
                 }
                 if (g == 0) c[0][0] = c0, c[0][1] = c1;
                 else c[1][0] = c0, c[1][1] = c1;
@@ -529,7 +537,7 @@ __global__ void __launch_bounds__(512) k_diaginv_block(const DiagItem* __restric
                 const int ea = We[row + 8 * g];
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
-                    const double2 p = fix_value(c[g][q], ea + Ce[col + 4 * q]);
+                    const double2 p = fix3_value(c[g][q], ea + Ce[col + 4 * q]);
                     double2& v = dst[(cq + 4 * q) * 8 + r8];
                     v = make_double2(v.x - p.x, v.y - p.y);
                 }
@@ -544,15 +552,15 @@ __global__ void __launch_bounds__(512) k_diaginv_block(const DiagItem* __restric
                 const int I = N0 + (u >= 2), J = N0 + (u >= 4);  // (0,0) (1,0) (1,1) of the pivot block
                 if (I >= nb8) continue;
                 const int row = (I - w8) * 8 + r8, c4 = cq + 4 * (u & 1), col = (J - w8) * 8 + c4;
-                FixSum c{};
+                Fix3Sum c{};
 #pragma unroll 2
-                for (int k = 0; k < kw; ++k) fix_mac(c, Wd[k * R + row], Cd[k * R + col]);
-                const double2 p = fix_value(c, We[row] + Ce[col]);
+                for (int k = 0; k < kw; ++k) fix3_mac(c, Wd[k * R + row], Cd[k * R + col]);
+                const double2 p = fix3_value(c, We[row] + Ce[col]);
                 double2& v = blk(I, J)[c4 * 8 + r8];
                 v = make_double2(v.x - p.x, v.y - p.y);
             }
             __syncthreads();
-            if (warp == wp) pivot(t + 1);
+            if (warp < 4) pivot(t + 1);
         }
         const int cnt = ctr[1];
         while (true) {

@@ -191,6 +191,7 @@ int run_phase(ndsi_plan* h, const Workspace& W, const SplitBuffers& SB, int phas
     // opt.split_slices; a smaller count fills and reads only the leading digits)
     const int ns = slices > 0 ? slices : P.opt.split_slices;
     const double pair_frac = split ? static_cast<double>(ns * (ns + 1)) / (P.opt.split_slices * (P.opt.split_slices + 1)) : 1.0;
+    size_t sliced = P.launches.size();  // the launch whose slices the buffers hold, none at first
     for (size_t li = 0; li < P.launches.size(); ++li) {
         const Launch& l = P.launches[li];
         if (l.phase != phase) continue;
@@ -205,8 +206,10 @@ int run_phase(ndsi_plan* h, const Workspace& W, const SplitBuffers& SB, int phas
                                    (h->prof.by_level ? ":L" + std::to_string(l.level) : std::string());
             e = timed(h->prof, "slice:" + tg, 0.0, h->SP.slice_bytes[si] * np, st, [&]() {
                 return split_slice_step(l, h->T.gemm_items, h->SP.d_items, h->SP.d_blocks, step, SB, ns,
-                                        bufs[l.bufA], strides[l.bufA], bufs[l.bufB], strides[l.bufB], np, st);
+                                        bufs[l.bufA], strides[l.bufA], bufs[l.bufB], strides[l.bufB], sliced + 1 == li,
+                                        np, st);
             });
+            sliced = li;
             if (e == cudaSuccess)
                 e = timed(
                     h->prof, "gemm_split:" + tg, l.flops * np, l.bytes * np, st,
@@ -282,14 +285,9 @@ int device_inputs(ndsi_plan* h, const double* H, const double* S, const double**
 int64_t bytes_per_pole(const ndsi_plan* h) {
     int64_t b = int64_t(16) * (h->P.front_total + h->P.scr_total);
     if (h->P.opt.precision == NDSI_PREC_SPLIT) {
-        int64_t a = 0, bb = 0, ea = 0, eb = 0;
-        for (const SplitStep& st : h->SP.steps) {
-            a = std::max<int64_t>(a, st.rowsA * st.Kcols);
-            bb = std::max<int64_t>(bb, st.rowsB * st.Kcols);
-            ea = std::max<int64_t>(ea, st.erowsA);
-            eb = std::max<int64_t>(eb, st.erowsB);
-        }
-        b += 2 * (a + bb) + 4 * (ea + eb);
+        int64_t el[4];
+        split_buffer_elements(h->SP.steps, el);
+        b += 2 * (el[0] + el[1]) + 4 * (el[2] + el[3]);
     }
     return b;
 }
@@ -338,10 +336,13 @@ static void build_split_metadata(ndsi_plan* h) {
         double sb = 0;
         for (int64_t i = 0; i < l.count; ++i) {
             const GemmItem& g = h->P.gemm_items[l.first + i];
-            // FP64 operand reads: once (one-pass slicer) or twice (two-pass)
-            sb += (st.slice_ldt > 0 ? 1.0 : 2.0) * 16.0 * (static_cast<double>(g.M) * g.K + static_cast<double>(g.N) * g.K);
+            // FP64 operand reads: once (one-pass slicer) or twice (two-pass); shared operands not at all
+            const double passes = (st.slice_ldt > 0 ? 1.0 : 2.0) * 16.0 * g.K;
+            if (!st.A.shared) sb += passes * g.M;
+            if (!st.B.shared) sb += passes * g.N;
         }
-        sb += 2.0 * (static_cast<double>(st.rowsA) + st.rowsB) * st.Kcols;
+        for (const SplitOperand* o : {&st.A, &st.B})
+            if (!o->shared) sb += 2.0 * static_cast<double>(o->rows) * o->Kcols;
         S.slice_bytes.push_back(sb);
         S.step_of_launch[li] = k++;
     }
@@ -954,8 +955,8 @@ int density_impl(ndsi_plan* h, const double* Hd, const double* Sd, const double*
     }
     if (h->graphs && !h->prof.on) {
         // replay the captured sweep; points and weights are read from zw / cw at run time
-        const std::vector<const void*> key = {Hd, Sd, rho_d, ne_d, e_d, h->W.fronts, h->W.scr, h->SB.sliceA,
-                                              h->SB.sliceB, h->cw, h->zw, h->cew, h->partials,
+        const std::vector<const void*> key = {Hd, Sd, rho_d, ne_d, e_d, h->W.fronts, h->W.scr, h->SB.slices[0],
+                                              h->SB.slices[1], h->cw, h->zw, h->cew, h->partials,
                                               reinterpret_cast<const void*>(static_cast<intptr_t>(nq)),
                                               reinterpret_cast<const void*>(static_cast<intptr_t>(chunk)),
                                               reinterpret_cast<const void*>(static_cast<intptr_t>(n_near))};

@@ -5,7 +5,8 @@
 // BF16 digits and FP32 tensor-core accumulation):
 //  * complex operands are stacked as real matrices: A'' = [Re A | Im A] (M x 2K) and, per
 //    NC-column tile of B, NC rows [Re B | -Im B] followed by NC rows [Im B | Re B], so that one
-//    real product gives Re C in the first NC accumulator columns and Im C in the next NC;
+//    real product gives Re C in the first NC accumulator columns and Im C in the next NC.  In memory
+//    a row is [Re | Im], of B [Re | Im | -Im], and a block of 64 elements is loaded from the part it needs;
 //  * every row of A'' (column of B) is scaled by a power of two 2^E with |x| < 2^E and written as
 //    S balanced base-256 digits, x = 2^(E-7) sum_t d_t 2^(-8(t-1)), d_1 in [-128,128],
 //    d_t in [-128,127]; digit t is stored pre-scaled, d_t 2^(-8(t-1)), exactly as BF16.  The
@@ -42,9 +43,9 @@
 // bounds it now is shared memory: a block's products read 360 KB of operands and the loads write
 // 156 KB, 4000 clocks at 128 bytes each against 3360 of tensor work.  Of the rest, 6% is the wait for
 // read-outs (with all six accumulators read every chunk: 20%) and 15% late loads.  Measured against
-// the two-stage form: 3D metallic lattice T = G_RR L_RJ 1435 -> 1557 TFLOP/s issued, Schur update
-// 1131 -> 1324; 3D cubic lattice 803 -> 1003 (Schur).  Tried without gain: a second producer thread
-// for B, L2 prefetches two blocks ahead (3% slower), 256-byte L2 promotion, giving the scales from 3
+// the two-stage form: 3D metallic lattice T = G_RR L_RJ 1435 -> 1519 TFLOP/s issued, Schur update
+// 1131 -> 1284; 3D cubic lattice 803 -> 967 (Schur); blocks that end with each part (below) cost
+// 2-4% of that.  Tried without gain: a second producer thread for B, L2 prefetches two blocks ahead (3% slower), 256-byte L2 promotion, giving the scales from 3
 // on back before the others.
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -67,29 +68,68 @@ void build_split_schedule(const Plan& P, int slices, const std::vector<int8_t>& 
     steps.clear();
     tiles.clear();
     blocks.clear();
+    // Launch li + 1 reads the rows that launch li slices as its other operand (the panel F_RJ of L_RJ =
+    // F_RJ A_J^{-1} and of the Schur update, L_RJ of both steps of the selected inversion): it takes
+    // those slices, which saves reading, converting and writing them a second time.  For that both
+    // operands have one format, K in blocks that end with the real and with the imaginary part (a
+    // part of 32 (mod 64) elements ends in a block of half the products), and a B row its digits once
+    // with one negated part instead of twice: 52 instead of 64 bytes an element for reading and
+    // writing.  80 poles of a cubic lattice of 16^3 atoms x 4 orbitals, slicing 75 -> 59 ms, GEMMs
+    // 140 -> 144 ms, all 268.5 -> 257.3 ms; a quarter of 160 poles of the 8-orbital lattice 725 -> 696 ms;
+    // twelve uneven systems, batched, 59.1 -> 56.9 ms.
+    auto shares = [&](size_t li, bool a_to_b) {
+        if (li + 1 >= P.launches.size()) return false;
+        const Launch &x = P.launches[li], &y = P.launches[li + 1];
+        if (!split_eligible(x) || !split_eligible(y) || x.phase != y.phase || x.count != y.count) return false;
+        if (a_to_b ? x.bufA != y.bufB || x.opA != OP_N || y.opB != OP_T || x.bufC == x.bufA
+                   : x.bufB != y.bufA || x.opB != OP_N || y.opA != OP_T || x.bufC == x.bufB)
+            return false;
+        for (int64_t i = 0; i < x.count; ++i) {
+            const GemmItem &g = P.gemm_items[x.first + i], &h = P.gemm_items[y.first + i];
+            if (a_to_b ? g.a_off != h.b_off || g.lda != h.ldb || g.M != h.N || g.K != h.K
+                       : g.b_off != h.a_off || g.ldb != h.lda || g.N != h.M || g.K != h.K)
+                return false;
+        }
+        return true;
+    };
+    bool takes_b = false, takes_a = false;  // this launch's B (A) operand is the previous launch's A (B)
     for (size_t li = 0; li < P.launches.size(); ++li) {
         const Launch& l = P.launches[li];
         if (!split_eligible(l)) continue;
         const int32_t nc = split_nc(slices, bands[li]);
         SplitStep st{};
         st.nc = nc;
+        const bool receives = takes_a || takes_b;
+        const bool gives_a = !receives && shares(li, true), gives_b = !receives && !gives_a && shares(li, false);
+        st.A.shared = takes_a;
+        st.B.shared = takes_b;
+        st.A.parts = gives_a ? 3 : 2;
+        st.B.parts = 3;
+        st.A.buf = gives_a || takes_a ? 1 : 0;
+        st.B.buf = 1 - st.A.buf;
         int32_t kmax = 0;
         st.tfirst = static_cast<int64_t>(tiles.size());
-        st.sa_first = static_cast<int64_t>(blocks.size());
+        st.A.first = static_cast<int64_t>(blocks.size());
         for (int64_t i = 0; i < l.count; ++i) {
             const GemmItem& g = P.gemm_items[l.first + i];
             SplitItem& s = items[l.first + i];
             s.Mpad = (g.M + kSplitBM - 1) / kSplitBM * kSplitBM;
             s.Npad = (g.N + nc - 1) / nc * nc;
             s.Kpad = (g.K + kSplitKB - 1) / kSplitKB * kSplitKB;
-            s.rowA = st.rowsA;
-            s.rowB = st.rowsB;
-            s.erowA = st.erowsA;
-            s.erowB = st.erowsB;
-            st.rowsA += static_cast<int64_t>(slices) * s.Mpad;
-            st.rowsB += static_cast<int64_t>(slices) * 2 * s.Npad;
-            st.erowsA += s.Mpad;
-            st.erowsB += s.Npad;
+            s.rowA = st.A.rows;
+            s.rowB = st.B.rows;
+            s.erowA = st.A.erows;
+            s.erowB = st.B.erows;
+            if (receives) {  // the layout of the launch before
+                const SplitItem& q = items[P.launches[li - 1].first + i];
+                (takes_b ? s.rowB : s.rowA) = takes_b ? q.rowA : q.rowB;
+                (takes_b ? s.erowB : s.erowA) = takes_b ? q.erowA : q.erowB;
+                (takes_b ? s.Npad : s.Mpad) = takes_b ? q.Mpad : q.Npad;
+            }
+            st.A.rows += static_cast<int64_t>(slices) * s.Mpad;
+            st.B.rows += static_cast<int64_t>(slices) * s.Npad;
+            st.A.erows += s.Mpad;
+            st.B.erows += s.Npad;
             kmax = std::max(kmax, s.Kpad);
             // Tile order.  The persistent CTAs take consecutive tiles, about kSplitConcurrentTiles
             // at a time, and move through K at about the same pace, so a K-block of an operand tile
@@ -101,7 +141,7 @@ void build_split_schedule(const Plan& P, int slices, const std::vector<int8_t>& 
             // streamed once per 128-row block (row-block order) read a 4000-wide L_RJ 9x over.
             const int32_t mt = (g.M + kSplitBM - 1) / kSplitBM, nt = (g.N + nc - 1) / nc;
             const double a_tile = static_cast<double>(slices) * 2.0 * s.Kpad * 2.0 * kSplitBM;
-            const double b_tile = static_cast<double>(slices) * 2.0 * s.Kpad * 2.0 * 2.0 * nc;
+            const double b_tile = static_cast<double>(slices) * 3.0 * s.Kpad * 2.0 * nc;
             // DRAM bytes of the order "groups of gp tiles along P swept across all q of Q"
             auto traffic = [&](int32_t gp, int32_t np_, int32_t nq, double p_tile, double q_tile) {
                 const double groups = std::ceil(static_cast<double>(np_) / gp);
@@ -161,16 +201,19 @@ void build_split_schedule(const Plan& P, int slices, const std::vector<int8_t>& 
             const GemmItem& g = P.gemm_items[l.first + i];
             for (int32_t r0 = 0; r0 < g.M; r0 += st.slice_rows) blocks.push_back(SliceBlock{static_cast<int32_t>(i), r0});
         }
-        st.sa_count = static_cast<int64_t>(blocks.size()) - st.sa_first;
-        st.sb_first = static_cast<int64_t>(blocks.size());
+        st.A.count = static_cast<int64_t>(blocks.size()) - st.A.first;
+        st.B.first = static_cast<int64_t>(blocks.size());
         for (int64_t i = 0; i < l.count; ++i) {
             const GemmItem& g = P.gemm_items[l.first + i];
             for (int32_t n0 = 0; n0 < g.N; n0 += st.slice_rows) blocks.push_back(SliceBlock{static_cast<int32_t>(i), n0});
         }
-        st.sb_count = static_cast<int64_t>(blocks.size()) - st.sb_first;
-        st.Kcols = std::max(64, 2 * kmax);
-        st.Kcols = (st.Kcols + 63) / 64 * 64;
+        st.B.count = static_cast<int64_t>(blocks.size()) - st.B.first;
+        auto cols = [&](int32_t parts) { return (std::max(64, parts * kmax) + 63) / 64 * 64; };
+        st.A.Kcols = takes_a ? steps.back().B.Kcols : cols(st.A.parts);
+        st.B.Kcols = takes_b ? steps.back().A.Kcols : cols(st.B.parts);
         steps.push_back(st);
+        takes_b = gives_a;
+        takes_a = gives_b;
     }
 }
 
@@ -499,7 +542,7 @@ struct SliceArgs {
     int32_t* expo;
     int64_t erows_pole;
     int rows, ldt;  // one-pass slicer: rows per block and shared-memory row stride
-    int nc;         // complex columns per output tile (B slices: groups of nc [Re|-Im], nc [Im|Re])
+    int parts;      // [Re | Im] or [Re | Im | -Im]
 };
 
 // Slices of one block of kSplitSliceRows rows of the stacked operand (A: rows m of op(A); B:
@@ -585,14 +628,7 @@ __global__ void __launch_bounds__(256, 3) k_slice(const SliceArgs p) {
             const int grow = blk.r0 + rr;
             if (grow >= nrows || col >= si.Kpad) continue;
             const int Er = rowmax[rr] < 0 ? -1021 : rowmax[rr] - 1022;
-            int64_t o0, ost;
-            if (!p.isB) {
-                o0 = pole * p.rows_pole + si.rowA + grow;
-                ost = si.Mpad;
-            } else {
-                o0 = pole * p.rows_pole + si.rowB + (grow / p.nc) * (2 * p.nc) + (grow % p.nc);
-                ost = 2 * si.Npad;
-            }
+            const int64_t o0 = pole * p.rows_pole + (p.isB ? si.rowB : si.rowA) + grow, ost = p.isB ? si.Npad : si.Mpad;
             const double2 v0 = tile[rr][kk];
             const double2 v1 = tile[rr][kk + 1];
             uint32_t wre[S], wim[S];
@@ -600,18 +636,11 @@ __global__ void __launch_bounds__(256, 3) k_slice(const SliceArgs p) {
             slice_pair<S>(v0.y, v1.y, Er, wim);
 #pragma unroll
             for (int t = 0; t < S; ++t) {
-                uint16_t* o1 = p.out + (o0 + t * ost) * p.Kcols;
-                if (!p.isB) {
-                    *reinterpret_cast<uint32_t*>(o1 + col) = wre[t];
-                    *reinterpret_cast<uint32_t*>(o1 + si.Kpad + col) = wim[t];
-                } else {
-                    // rows [Re | -Im] and [Im | Re]; negation flips the BF16 sign bits
-                    uint16_t* o2 = o1 + p.nc * static_cast<int64_t>(p.Kcols);
-                    *reinterpret_cast<uint32_t*>(o1 + col) = wre[t];
-                    *reinterpret_cast<uint32_t*>(o1 + si.Kpad + col) = wim[t] ^ 0x80008000u;
-                    *reinterpret_cast<uint32_t*>(o2 + col) = wim[t];
-                    *reinterpret_cast<uint32_t*>(o2 + si.Kpad + col) = wre[t];
-                }
+                uint16_t* o = p.out + (o0 + t * ost) * p.Kcols + col;
+                *reinterpret_cast<uint32_t*>(o) = wre[t];
+                *reinterpret_cast<uint32_t*>(o + si.Kpad) = wim[t];
+                // negation flips the BF16 sign bits
+                if (p.parts == 3) *reinterpret_cast<uint32_t*>(o + 2 * si.Kpad) = wim[t] ^ 0x80008000u;
             }
         }
         __syncthreads();
@@ -688,14 +717,7 @@ __global__ void __launch_bounds__(256) k_slice1(const SliceArgs p) {
         const int grow = blk.r0 + rr;
         if (grow >= nrows) continue;
         const int Er = rowmax[rr] < 0 ? -1021 : rowmax[rr] - 1022;
-        int64_t o0, ost;
-        if (!p.isB) {
-            o0 = pole * p.rows_pole + si.rowA + grow;
-            ost = si.Mpad;
-        } else {
-            o0 = pole * p.rows_pole + si.rowB + (grow / p.nc) * (2 * p.nc) + (grow % p.nc);
-            ost = 2 * si.Npad;
-        }
+        const int64_t o0 = pole * p.rows_pole + (p.isB ? si.rowB : si.rowA) + grow, ost = p.isB ? si.Npad : si.Mpad;
         const double2 v0 = kk < K ? t1[rr * ldt + kk] : make_double2(0.0, 0.0);
         const double2 v1 = kk + 1 < K ? t1[rr * ldt + kk + 1] : make_double2(0.0, 0.0);
         uint32_t wre[S], wim[S];
@@ -703,18 +725,11 @@ __global__ void __launch_bounds__(256) k_slice1(const SliceArgs p) {
         slice_pair<S>(v0.y, v1.y, Er, wim);
 #pragma unroll
         for (int t = 0; t < S; ++t) {
-            uint16_t* o1 = p.out + (o0 + t * ost) * p.Kcols;
-            if (!p.isB) {
-                *reinterpret_cast<uint32_t*>(o1 + kk) = wre[t];
-                *reinterpret_cast<uint32_t*>(o1 + si.Kpad + kk) = wim[t];
-            } else {
-                // rows [Re | -Im] and [Im | Re]; negation flips the BF16 sign bits
-                uint16_t* o2 = o1 + p.nc * static_cast<int64_t>(p.Kcols);
-                *reinterpret_cast<uint32_t*>(o1 + kk) = wre[t];
-                *reinterpret_cast<uint32_t*>(o1 + si.Kpad + kk) = wim[t] ^ 0x80008000u;
-                *reinterpret_cast<uint32_t*>(o2 + kk) = wim[t];
-                *reinterpret_cast<uint32_t*>(o2 + si.Kpad + kk) = wre[t];
-            }
+            uint16_t* o = p.out + (o0 + t * ost) * p.Kcols + kk;
+            *reinterpret_cast<uint32_t*>(o) = wre[t];
+            *reinterpret_cast<uint32_t*>(o + si.Kpad) = wim[t];
+            // negation flips the BF16 sign bits
+            if (p.parts == 3) *reinterpret_cast<uint32_t*>(o + 2 * si.Kpad) = wim[t] ^ 0x80008000u;
         }
     }
     if (tid < R && blk.r0 + tid < nrows) {
@@ -849,7 +864,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int64_t n_work = p.tcount * p.np;
     int* claim = p.status + 2;  // [0] items claimed beyond the first wave, [1] CTAs finished
     auto tile_of = [&](int64_t w) { return p.tiles[p.tfirst + w % p.tcount]; };
-    auto nkb_of = [&](const GemmTile& t) { return 2 * p.sitems[p.ifirst + t.item].Kpad / kSplitStageK; };
+    // blocks of up to kSplitStageK elements of A's real part, then as many of its imaginary part
+    auto kpad_of = [&](const GemmTile& t) { return p.sitems[p.ifirst + t.item].Kpad; };
+    auto nkh_of = [](int kpad) { return (kpad + kSplitStageK - 1) / kSplitStageK; };
 
     if (threadIdx.x == 0) {
 #pragma unroll
@@ -893,25 +910,30 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const GemmTile tile = tile_of(w);
                 const int64_t pole = w / p.tcount;
                 const SplitItem si = p.sitems[p.ifirst + tile.item];
-                const int nkb = nkb_of(tile);
+                const int nkh = nkh_of(si.Kpad), nkb = 2 * nkh;
                 const int yA0 = static_cast<int>(pole * p.rowsA + si.rowA + tile.m0);
-                const int yB0 = static_cast<int>(pole * p.rowsB + si.rowB + (tile.n0 / NC) * NB);
+                const int yB0 = static_cast<int>(pole * p.rowsB + si.rowB + tile.n0);
                 bool ok = true;
                 for (int kb = 0; kb < nkb && ok; ++kb) {
-                    const int x = kb * kSplitStageK;
+                    const bool im = kb >= nkh;
+                    const int k = (im ? kb - nkh : kb) * kSplitStageK;
+                    // parts of A, of B for the real and of B for the imaginary output columns
+                    const int xa = im ? si.Kpad + k : k, xr = im ? 2 * si.Kpad + k : k, xi = im ? k : si.Kpad + k;
                     auto load_a = [&](int t) {
                         if (!ok || !(ok = slot_free(a_empty, ia, NA))) return;
                         const int sl = static_cast<int>(ia++ % NA);
                         mbar_expect_tx(&a_full[sl], kTileBytes);
-                        tma_load_2d(smem + sl * kTileBytes, &tmA, x, yA0 + t * si.Mpad, &a_full[sl]);
+                        tma_load_2d(smem + sl * kTileBytes, &tmA, xa, yA0 + t * si.Mpad, &a_full[sl]);
                     };
                     auto load_b = [&](int u0, int u1) {  // digits u0 .. u1-1 into consecutive rows of one group
                         if (!ok || !(ok = slot_free(b_empty, ib, NG))) return;
                         const int sl = static_cast<int>(ib++ % NG);
                         mbar_expect_tx(&b_full[sl], (u1 - u0) * kTileB);
-                        for (int u = u0; u < u1; ++u)
-                            tma_load_2d(b_ring + sl * Ring::GROUP + (u - u0) * kTileB, &tmB, x, yB0 + u * 2 * si.Npad,
-                                        &b_full[sl]);
+                        for (int u = u0; u < u1; ++u) {
+                            uint8_t* dst = b_ring + sl * Ring::GROUP + (u - u0) * kTileB;
+                            tma_load_2d(dst, &tmB, xr, yB0 + u * si.Npad, &b_full[sl]);
+                            tma_load_2d(dst + kTileB / 2, &tmB, xi, yB0 + u * si.Npad, &b_full[sl]);
+                        }
                     };
                     if constexpr (EXACT) {
                         load_b(G, S);                                    // high digits, needed first
@@ -945,10 +967,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int64_t w = tq[slot];
                 mbar_arrive(&tq_empty[slot]);
                 if (w < 0) break;
-                const int nkb = nkb_of(tile_of(w));
+                const int kpad = kpad_of(tile_of(w)), nkh = nkh_of(kpad), nkb = 2 * nkh;
                 uint32_t keep = 0;  // scales whose accumulators hold sums of earlier chunks of the tile
                 for (int kb = 0; kb < nkb && ok; ++kb) {
                     const bool first_in_chunk = (kb % kSplitChunkKB) == 0;
+                    // K16 steps of the block: the last one of either part has 2 or 4
+                    const int steps = (kpad - (kb >= nkh ? kb - nkh : kb) * kSplitStageK) / 16;
                     if (first_in_chunk && c > 0) {
                         if (!(ok = mbar_wait(tmem_free, static_cast<uint32_t>((c - 1) & 1), abort))) break;
                     }
@@ -967,77 +991,82 @@ __global__ void __launch_bounds__(kThreads, 1)
                         ok = ok && mbar_wait(&b_full[i % NG], static_cast<uint32_t>((i / NG) & 1), abort);
                         return sdesc_sw(smem_u32(b_ring + (i % NG) * Ring::GROUP));
                     };
-                    if constexpr (EXACT) {
-                        // A_t times digits u0 .. u0+n-1 of a group: one MMA per K16 step into the
-                        // accumulators of scales t+u0 .. t+u0+n-1; the first products of a chunk go
-                        // scale by scale, each starting or continuing its own sum
-                        auto products = [&](int t, int u0, int n, uint64_t db) {
-                            const uint32_t d = tmem + (t + u0) * NB;
+                    auto block = [&](auto nsteps) {
+                        constexpr int STEPS = decltype(nsteps)::value;
+                        if constexpr (EXACT) {
+                            // A_t times digits u0 .. u0+n-1 of a group: one MMA per K16 step into the
+                            // accumulators of scales t+u0 .. t+u0+n-1; the first products of a chunk go
+                            // scale by scale, each starting or continuing its own sum
+                            auto products = [&](int t, int u0, int n, uint64_t db) {
+                                const uint32_t d = tmem + (t + u0) * NB;
 #pragma unroll
-                            for (int ks = 0; ks < kK16Steps; ++ks) {
-                                const uint64_t a = da[t] + static_cast<uint64_t>((ks * 32) >> 4);
-                                const uint64_t b = db + static_cast<uint64_t>((ks * 32) >> 4);
-                                if (t == 0 && ks == 0 && first_in_chunk) {
+                                for (int ks = 0; ks < STEPS; ++ks) {
+                                    const uint64_t a = da[t] + static_cast<uint64_t>((ks * 32) >> 4);
+                                    const uint64_t b = db + static_cast<uint64_t>((ks * 32) >> 4);
+                                    if (t == 0 && ks == 0 && first_in_chunk) {
 #pragma unroll
-                                    for (int u = 0; u < G; ++u)
-                                        if (u < n)
-                                            umma_bf16(d + u * NB, a, b + static_cast<uint64_t>((u * kTileB) >> 4),
-                                                      idesc_bf16(NB), (keep >> (u0 + u)) & 1u);
-                                } else {
-                                    umma_bf16(d, a, b, idesc_bf16(static_cast<uint32_t>(n * NB)), 1u);
+                                        for (int u = 0; u < G; ++u)
+                                            if (u < n)
+                                                umma_bf16(d + u * NB, a, b + static_cast<uint64_t>((u * kTileB) >> 4),
+                                                          idesc_bf16(NB), (keep >> (u0 + u)) & 1u);
+                                    } else {
+                                        umma_bf16(d, a, b, idesc_bf16(static_cast<uint32_t>(n * NB)), 1u);
+                                    }
                                 }
+                            };
+                            const uint64_t bh = wait_b(0);
+#pragma unroll
+                            for (int t = 0; t < S - G; ++t) {
+                                wait_a(t);
+                                if (!ok) break;
+                                tc_fence_after();
+                                products(t, G, S - G - t, bh);
                             }
-                        };
-                        const uint64_t bh = wait_b(0);
+                            if (!ok) return;
+                            umma_commit(&b_empty[ib % NG]);
+                            const uint64_t bl = wait_b(1);
 #pragma unroll
-                        for (int t = 0; t < S - G; ++t) {
-                            wait_a(t);
-                            if (!ok) break;
-                            tc_fence_after();
-                            products(t, G, S - G - t, bh);
-                        }
-                        if (!ok) break;
-                        umma_commit(&b_empty[ib % NG]);
-                        const uint64_t bl = wait_b(1);
-#pragma unroll
-                        for (int t = 0; t < S; ++t) {
-                            if (t >= S - G) wait_a(t);
-                            if (!ok) break;
-                            tc_fence_after();
-                            products(t, 0, S - t < G ? S - t : G, bl);
-                            free_a(t);
-                        }
-                        if (!ok) break;
-                        umma_commit(&b_empty[(ib + 1) % NG]);
-                    } else {
-                        // bands 0..BANDS-2 hold one scale each, band BANDS-1 the rest; digit u is group
-                        // S-1-u of the block and free once A_{S-1-u} has met it
-                        uint64_t db[S];
-#pragma unroll
-                        for (int u = S - 1; u >= 0; --u) db[u] = wait_b(S - 1 - u);
-#pragma unroll
-                        for (int t = 0; t < S; ++t) {
-                            wait_a(t);
-                            if (!ok) break;
-                            tc_fence_after();
-#pragma unroll
-                            for (int u = S - 1; u >= 0; --u) {
-                                if (t + u > S - 1) continue;
-                                constexpr int last = BANDS - 1;
-                                const int band = t + u < last ? t + u : last;
-                                // the first product into a band: t == 0, and for the tail the first u
-                                const bool lead = t == 0 && (t + u < last || u == S - 1);
-#pragma unroll
-                                for (int ks = 0; ks < kK16Steps; ++ks)
-                                    umma_bf16(tmem + band * NB, da[t] + static_cast<uint64_t>((ks * 32) >> 4),
-                                              db[u] + static_cast<uint64_t>((ks * 32) >> 4), idesc_bf16(NB),
-                                              lead && ks == 0 && first_in_chunk ? 0u : 1u);
+                            for (int t = 0; t < S; ++t) {
+                                if (t >= S - G) wait_a(t);
+                                if (!ok) break;
+                                tc_fence_after();
+                                products(t, 0, S - t < G ? S - t : G, bl);
+                                free_a(t);
                             }
-                            free_a(t);
-                            umma_commit(&b_empty[(ib + t) % NG]);
+                            if (!ok) return;
+                            umma_commit(&b_empty[(ib + 1) % NG]);
+                        } else {
+                            // bands 0..BANDS-2 hold one scale each, band BANDS-1 the rest; digit u is group
+                            // S-1-u of the block and free once A_{S-1-u} has met it
+                            uint64_t db[S];
+#pragma unroll
+                            for (int u = S - 1; u >= 0; --u) db[u] = wait_b(S - 1 - u);
+#pragma unroll
+                            for (int t = 0; t < S; ++t) {
+                                wait_a(t);
+                                if (!ok) break;
+                                tc_fence_after();
+#pragma unroll
+                                for (int u = S - 1; u >= 0; --u) {
+                                    if (t + u > S - 1) continue;
+                                    constexpr int last = BANDS - 1;
+                                    const int band = t + u < last ? t + u : last;
+                                    // the first product into a band: t == 0, and for the tail the first u
+                                    const bool lead = t == 0 && (t + u < last || u == S - 1);
+#pragma unroll
+                                    for (int ks = 0; ks < STEPS; ++ks)
+                                        umma_bf16(tmem + band * NB, da[t] + static_cast<uint64_t>((ks * 32) >> 4),
+                                                  db[u] + static_cast<uint64_t>((ks * 32) >> 4), idesc_bf16(NB),
+                                                  lead && ks == 0 && first_in_chunk ? 0u : 1u);
+                                }
+                                free_a(t);
+                                umma_commit(&b_empty[(ib + t) % NG]);
+                            }
                         }
-                        if (!ok) break;
-                    }
+                    };
+                    if (steps >= kK16Steps) block(std::integral_constant<int, kK16Steps>{});
+                    else block(std::integral_constant<int, kK16Steps / 2>{});
+                    if (!ok) break;
                     ia += S;
                     ib += PER;
                     const bool last_kb = kb == nkb - 1;
@@ -1082,7 +1111,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int64_t pole = w / p.tcount;
             const GemmItem it = p.items[p.ifirst + tile.item];
             const SplitItem si = p.sitems[p.ifirst + tile.item];
-            const int nchunks = (nkb_of(tile) + kSplitChunkKB - 1) / kSplitChunkKB;
+            const int nchunks = (2 * nkh_of(kpad_of(tile)) + kSplitChunkKB - 1) / kSplitChunkKB;
             double2* Cp = p.C + pole * p.sC + it.c_off;
             if (et < 128) {
                 const int m = tile.m0 + et;
@@ -1301,10 +1330,10 @@ cudaError_t split_init() {
 }
 
 void split_free(SplitBuffers& B) {
-    if (B.sliceA) cudaFree(B.sliceA);
-    if (B.sliceB) cudaFree(B.sliceB);
-    if (B.expA) cudaFree(B.expA);
-    if (B.expB) cudaFree(B.expB);
+    for (int i = 0; i < 2; ++i) {
+        if (B.slices[i]) cudaFree(B.slices[i]);
+        if (B.expo[i]) cudaFree(B.expo[i]);
+    }
     B = SplitBuffers{};
 }
 
@@ -1320,35 +1349,35 @@ static cudaError_t encode(CUtensorMap* map, void* base, int64_t cols, int64_t ro
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+void split_buffer_elements(const std::vector<SplitStep>& steps, int64_t out[4]) {
+    for (int i = 0; i < 4; ++i) out[i] = 0;
+    for (const SplitStep& s : steps)
+        for (const SplitOperand* o : {&s.A, &s.B}) {
+            out[o->buf] = std::max<int64_t>(out[o->buf], o->rows * o->Kcols);
+            out[2 + o->buf] = std::max<int64_t>(out[2 + o->buf], o->erows);
+        }
+}
+
 cudaError_t split_alloc(SplitBuffers& B, const std::vector<SplitStep>& steps, int slices, int np) {
     (void)slices;
-    size_t ca = 0, cb = 0, cea = 0, ceb = 0;
-    for (const SplitStep& s : steps) {
-        ca = std::max(ca, static_cast<size_t>(s.rowsA) * s.Kcols * np);
-        cb = std::max(cb, static_cast<size_t>(s.rowsB) * s.Kcols * np);
-        cea = std::max(cea, static_cast<size_t>(s.erowsA) * np);
-        ceb = std::max(ceb, static_cast<size_t>(s.erowsB) * np);
-    }
-    if (B.np >= np && B.capA >= ca && B.capB >= cb && !B.tmA.empty()) return cudaSuccess;
+    int64_t el[4];
+    split_buffer_elements(steps, el);
+    const size_t cap[2] = {static_cast<size_t>(el[0]) * np, static_cast<size_t>(el[1]) * np};
+    if (B.np >= np && B.cap[0] >= cap[0] && B.cap[1] >= cap[1] && !B.tmA.empty()) return cudaSuccess;
     split_free(B);
     cudaError_t e;
-    if ((e = cudaMalloc(&B.sliceA, std::max<size_t>(ca, 64) * 2)) != cudaSuccess) return e;
-    if ((e = cudaMalloc(&B.sliceB, std::max<size_t>(cb, 64) * 2)) != cudaSuccess) return e;
-    if ((e = cudaMalloc(&B.expA, std::max<size_t>(cea, 1) * 4)) != cudaSuccess) return e;
-    if ((e = cudaMalloc(&B.expB, std::max<size_t>(ceb, 1) * 4)) != cudaSuccess) return e;
-    B.capA = ca;
-    B.capB = cb;
-    B.capEA = cea;
-    B.capEB = ceb;
+    for (int i = 0; i < 2; ++i) {
+        if ((e = cudaMalloc(&B.slices[i], std::max<size_t>(cap[i], 64) * 2)) != cudaSuccess) return e;
+        if ((e = cudaMalloc(&B.expo[i], std::max<size_t>(static_cast<size_t>(el[2 + i]) * np, 1) * 4)) != cudaSuccess) return e;
+        B.cap[i] = cap[i];
+    }
     B.np = np;
     B.tmA.assign(steps.size(), CUtensorMap{});
     B.tmB.assign(steps.size(), CUtensorMap{});
     for (size_t i = 0; i < steps.size(); ++i) {
         const SplitStep& s = steps[i];
-        if ((e = encode(&B.tmA[i], B.sliceA, s.Kcols, std::max<int64_t>(s.rowsA * np, 128), kSplitBM)) != cudaSuccess)
-            return e;
-        if ((e = encode(&B.tmB[i], B.sliceB, s.Kcols, std::max<int64_t>(s.rowsB * np, 128), 2 * s.nc)) != cudaSuccess)
-            return e;
+        if ((e = encode(&B.tmA[i], B.slices[s.A.buf], s.A.Kcols, s.A.rows * np, kSplitBM)) != cudaSuccess) return e;
+        if ((e = encode(&B.tmB[i], B.slices[s.B.buf], s.B.Kcols, s.B.rows * np, s.nc)) != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
@@ -1356,25 +1385,22 @@ cudaError_t split_alloc(SplitBuffers& B, const std::vector<SplitStep>& steps, in
 template <int S>
 static cudaError_t run_slice(const Launch& l, const GemmItem* items_dev, const SplitItem* sitems_dev,
                              const SliceBlock* blocks_dev, const SplitStep& step, const SplitBuffers& B,
-                             const double2* Abuf, int64_t sA, const double2* Bbuf, int64_t sB, int np,
+                             const double2* Abuf, int64_t sA, const double2* Bbuf, int64_t sB, bool ready, int np,
                              cudaStream_t st) {
-    SliceArgs sa{items_dev, sitems_dev, blocks_dev, step.sa_first, l.first, Abuf, sA, l.opA, 0,
-                 B.sliceA, step.rowsA, step.Kcols, B.expA, step.erowsA, step.slice_rows, step.slice_ldt, step.nc};
-    SliceArgs sb{items_dev, sitems_dev, blocks_dev, step.sb_first, l.first, Bbuf, sB, l.opB, 1,
-                 B.sliceB, step.rowsB, step.Kcols, B.expB, step.erowsB, step.slice_rows, step.slice_ldt, step.nc};
-    if (step.slice_ldt > 0) {
+    for (int isB = 0; isB < 2; ++isB) {
+        const SplitOperand& o = isB ? step.B : step.A;
+        if (o.shared && ready) continue;
+        const SliceArgs a{items_dev, sitems_dev, blocks_dev, o.first, l.first, isB ? Bbuf : Abuf, isB ? sB : sA,
+                          isB ? l.opB : l.opA, isB, B.slices[o.buf], o.rows, o.Kcols, B.expo[o.buf], o.erows,
+                          step.slice_rows, step.slice_ldt, o.parts};
+        const dim3 grid(static_cast<unsigned>(o.count), np);
         const size_t sm = static_cast<size_t>(step.slice_rows) * step.slice_ldt * sizeof(double2);
-        k_slice1<S><<<dim3(static_cast<unsigned>(step.sa_count), np), 256, sm, st>>>(sa);
-        cudaError_t e = cudaGetLastError();
+        if (step.slice_ldt > 0) k_slice1<S><<<grid, 256, sm, st>>>(a);
+        else k_slice<S><<<grid, 256, 0, st>>>(a);
+        const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        k_slice1<S><<<dim3(static_cast<unsigned>(step.sb_count), np), 256, sm, st>>>(sb);
-        return cudaGetLastError();
     }
-    k_slice<S><<<dim3(static_cast<unsigned>(step.sa_count), np), 256, 0, st>>>(sa);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_slice<S><<<dim3(static_cast<unsigned>(step.sb_count), np), 256, 0, st>>>(sb);
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
 template <int S>
@@ -1383,8 +1409,8 @@ static cudaError_t run_mma(const Launch& l, int step_index, const GemmItem* item
                            const SplitBuffers& B, double2* Cbuf, int64_t sC, int np, int* status,
                            cudaStream_t st) {
     if ((l.alpha != 1.0 && l.alpha != -1.0) || (l.beta != 0.0 && l.beta != 1.0)) return cudaErrorInvalidValue;
-    const GemmArgs ga{items_dev, sitems_dev, stiles_dev, step.tfirst, l.first, step.rowsA, step.rowsB,
-                      step.erowsA, step.erowsB, B.expA, B.expB, Cbuf, sC, l.alpha < 0 ? 1 : 0, l.beta != 0.0 ? 1 : 0,
+    const GemmArgs ga{items_dev, sitems_dev, stiles_dev, step.tfirst, l.first, step.A.rows, step.B.rows,
+                      step.A.erows, step.B.erows, B.expo[step.A.buf], B.expo[step.B.buf], Cbuf, sC, l.alpha < 0 ? 1 : 0, l.beta != 0.0 ? 1 : 0,
                       l.lower, status, step.tcount, np};
     const int64_t work = step.tcount * np;
     const unsigned grid = static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>(work, g_num_sms)));
@@ -1409,12 +1435,12 @@ static cudaError_t run_mma(const Launch& l, int step_index, const GemmItem* item
 cudaError_t split_slice_step(const Launch& l, const GemmItem* items_dev, const SplitItem* sitems_dev,
                              const SliceBlock* blocks_dev, const SplitStep& step, const SplitBuffers& B,
                              int slices, const double2* Abuf, int64_t sA, const double2* Bbuf, int64_t sB,
-                             int np, cudaStream_t st) {
+                             bool ready, int np, cudaStream_t st) {
     switch (slices) {
-        case 4: return run_slice<4>(l, items_dev, sitems_dev, blocks_dev, step, B, Abuf, sA, Bbuf, sB, np, st);
-        case 5: return run_slice<5>(l, items_dev, sitems_dev, blocks_dev, step, B, Abuf, sA, Bbuf, sB, np, st);
-        case 6: return run_slice<6>(l, items_dev, sitems_dev, blocks_dev, step, B, Abuf, sA, Bbuf, sB, np, st);
-        case 7: return run_slice<7>(l, items_dev, sitems_dev, blocks_dev, step, B, Abuf, sA, Bbuf, sB, np, st);
+        case 4: return run_slice<4>(l, items_dev, sitems_dev, blocks_dev, step, B, Abuf, sA, Bbuf, sB, ready, np, st);
+        case 5: return run_slice<5>(l, items_dev, sitems_dev, blocks_dev, step, B, Abuf, sA, Bbuf, sB, ready, np, st);
+        case 6: return run_slice<6>(l, items_dev, sitems_dev, blocks_dev, step, B, Abuf, sA, Bbuf, sB, ready, np, st);
+        case 7: return run_slice<7>(l, items_dev, sitems_dev, blocks_dev, step, B, Abuf, sA, Bbuf, sB, ready, np, st);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -42,23 +42,32 @@ constexpr double kSplitFarRatio = 32.0;
 
 // Where an item's slices and exponents live inside one pole's block of the step buffers.
 struct SplitItem {
-    int64_t rowA, rowB;     // first slice row of the item (A: S*Mpad rows, B: S*2*Npad rows)
+    int64_t rowA, rowB;     // first slice row of the item's operand (digit t at row + t Mpad, + t Npad)
     int64_t erowA, erowB;   // first exponent of the item
-    int32_t Mpad, Npad;     // Mpad multiple of 128 rows, Npad multiple of nc complex columns
+    int32_t Mpad, Npad;     // slice rows per digit: at least the tiles' 128 rows, nc complex columns
     int32_t Kpad, pad;      // multiple of kSplitKB (complex K); stacked K is 2*Kpad
+};
+
+// Slices of one operand of a step.  A slice row holds the digits of one row of op(A) or column of op(B):
+// parts [Re | Im] of Kpad elements each, and [Re | Im | -Im] for a B operand, whose real and imaginary
+// output columns take (Re, -Im) and (Im, Re) of the same rows against A's (Re, Im).
+struct SplitOperand {
+    int64_t rows, erows;                   // per pole
+    int32_t Kcols;                         // row length of the slice buffer
+    int32_t parts;                         // 2 or 3
+    int32_t buf;                           // slice buffer 0 or 1
+    int32_t shared;                        // rows are those of the previous launch's other operand
+    int64_t first, count;                  // slicing blocks in the block list
 };
 
 // Per GEMM launch: sizes of one pole's block in the step buffers, and the split tile range.
 struct SplitStep {
-    int64_t rowsA, rowsB, erowsA, erowsB;  // per pole
-    int32_t Kcols;                         // row length of the slice buffers (2*max Kpad)
+    SplitOperand A, B;
     int32_t nc;                            // complex columns per output tile (64, 48, 40 or 32)
     int32_t slice_rows;                    // operand rows per slicing block
     int32_t slice_ldt;                     // one-pass slicing: shared-memory row stride (0: two passes)
     int32_t pad;
     int64_t tfirst, tcount;                // tiles in the split tile list
-    int64_t sa_first, sa_count;            // slicing blocks of A (rows of op(A)) in the block list
-    int64_t sb_first, sb_count;            // slicing blocks of B (columns of op(B))
 };
 
 // A slicing block: item (relative to the launch) and its first row (A) or complex column (B).
@@ -73,26 +82,27 @@ void build_split_schedule(const Plan& P, int slices, const std::vector<int8_t>& 
                           std::vector<GemmTile>& tiles, std::vector<SliceBlock>& blocks);
 
 struct SplitBuffers {
-    uint16_t* sliceA = nullptr;   // bf16 bit patterns
-    uint16_t* sliceB = nullptr;
-    int32_t* expA = nullptr;
-    int32_t* expB = nullptr;
-    size_t capA = 0, capB = 0, capEA = 0, capEB = 0;  // elements
+    uint16_t* slices[2] = {};     // bf16 bit patterns
+    int32_t* expo[2] = {};
+    size_t cap[2] = {};           // slice elements
     std::vector<CUtensorMap> tmA, tmB;                // one per split step (for np_cap poles)
     int32_t np = 0;
 };
 
+// Slice elements (out[0], out[1]) and exponents (out[2], out[3]) of the two buffers for one pole.
+void split_buffer_elements(const std::vector<SplitStep>& steps, int64_t out[4]);
 cudaError_t split_init();
 // Allocate the slice buffers for np poles and encode the tensor maps of every step.
 cudaError_t split_alloc(SplitBuffers& B, const std::vector<SplitStep>& steps, int slices, int np);
 void split_free(SplitBuffers& B);
 
-// One GEMM launch of the schedule in split precision: slice A and B (split_slice_step), then the
-// tensor-core product and FP64 epilogue (split_mma_step).
+// One GEMM launch of the schedule in split precision: slice A and B (split_slice_step; a shared operand
+// only when its slices are not `ready` from the previous launch), then the tensor-core product and
+// FP64 epilogue (split_mma_step).
 cudaError_t split_slice_step(const Launch& l, const GemmItem* items_dev, const SplitItem* sitems_dev,
                              const SliceBlock* blocks_dev, const SplitStep& step, const SplitBuffers& B,
                              int slices, const double2* Abuf, int64_t sA, const double2* Bbuf, int64_t sB,
-                             int np, cudaStream_t st);
+                             bool ready, int np, cudaStream_t st);
 cudaError_t split_mma_step(const Launch& l, int step_index, const GemmItem* items_dev,
                            const SplitItem* sitems_dev, const GemmTile* stiles_dev, const SplitStep& step,
                            const SplitBuffers& B, int slices, double2* Cbuf, int64_t sC, int np, int* status,

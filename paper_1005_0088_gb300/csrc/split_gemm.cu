@@ -45,8 +45,8 @@
 // read-outs (with all six accumulators read every chunk: 20%) and 15% late loads.  Measured against
 // the two-stage form: 3D metallic lattice T = G_RR L_RJ 1435 -> 1519 TFLOP/s issued, Schur update
 // 1131 -> 1284; 3D cubic lattice 803 -> 967 (Schur); blocks that end with each part (below) cost
-// 2-4% of that.  Tried without gain: a second producer thread for B, L2 prefetches two blocks ahead (3% slower), 256-byte L2 promotion, giving the scales from 3
-// on back before the others.
+// 2-4% of that.  Tried without gain: a second producer thread for B, L2 prefetches two blocks ahead (3%
+// slower), 256-byte L2 promotion, giving the scales from 3 on back before the others.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_runtime.h>

@@ -191,10 +191,11 @@ int run_phase(ndsi_plan* h, const Workspace& W, const SplitBuffers& SB, int phas
     // opt.split_slices; a smaller count fills and reads only the leading digits)
     const int ns = slices > 0 ? slices : P.opt.split_slices;
     const double pair_frac = split ? static_cast<double>(ns * (ns + 1)) / (P.opt.split_slices * (P.opt.split_slices + 1)) : 1.0;
-    size_t sliced = P.launches.size();  // the launch whose slices the buffers hold, none at first
+    // the launch whose slices the buffers hold, and the copy that a slicer has done: none at first
+    size_t sliced = P.launches.size(), copied = P.launches.size();
     for (size_t li = 0; li < P.launches.size(); ++li) {
         const Launch& l = P.launches[li];
-        if (l.phase != phase) continue;
+        if (l.phase != phase || li == copied) continue;
         cudaError_t e;
         h->prof.cur_launch = static_cast<int64_t>(li);
         if (split && split_eligible(l) && h->SP.use_split[li]) {
@@ -204,10 +205,16 @@ int run_phase(ndsi_plan* h, const Workspace& W, const SplitBuffers& SB, int phas
             const int64_t strides[2] = {W.front_stride, W.scr_stride};
             const std::string tg = std::string(tag_name(l.tag)) +
                                    (h->prof.by_level ? ":L" + std::to_string(l.level) : std::string());
+            const bool ready = sliced + 1 == li;
+            SplitCopy copy;
+            if (ready && step.fuse_copy) {
+                const Launch& c = P.launches[li + 1];
+                copy = SplitCopy{h->T.copy_items + c.first, W.fronts, W.front_stride, c.alpha};
+                copied = li + 1;
+            }
             e = timed(h->prof, "slice:" + tg, 0.0, h->SP.slice_bytes[si] * np, st, [&]() {
                 return split_slice_step(l, h->T.gemm_items, h->SP.d_items, h->SP.d_blocks, step, SB, ns,
-                                        bufs[l.bufA], strides[l.bufA], bufs[l.bufB], strides[l.bufB], sliced + 1 == li,
-                                        np, st);
+                                        bufs[l.bufA], strides[l.bufA], bufs[l.bufB], strides[l.bufB], ready, copy, np, st);
             });
             sliced = li;
             if (e == cudaSuccess)

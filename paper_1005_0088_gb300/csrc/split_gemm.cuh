@@ -66,7 +66,7 @@ struct SplitStep {
     int32_t nc;                            // complex columns per output tile (64, 48, 40 or 32)
     int32_t slice_rows;                    // operand rows per slicing block
     int32_t slice_ldt;                     // one-pass slicing: shared-memory row stride (0: two passes)
-    int32_t pad;
+    int32_t fuse_copy;                     // the next launch copies this step's own sliced operand
     int64_t tfirst, tcount;                // tiles in the split tile list
 };
 
@@ -98,11 +98,18 @@ void split_free(SplitBuffers& B);
 
 // One GEMM launch of the schedule in split precision: slice A and B (split_slice_step; a shared operand
 // only when its slices are not `ready` from the previous launch), then the tensor-core product and
-// FP64 epilogue (split_mma_step).
+// FP64 epilogue (split_mma_step).  With `copy` the slicer of the operand that is not
+// shared also writes it to its place in the fronts (the schedule's next launch, SplitStep::fuse_copy).
+struct SplitCopy {
+    const CopyItem* items = nullptr;
+    double2* dst = nullptr;
+    int64_t stride = 0;
+    double scale = 1.0;
+};
 cudaError_t split_slice_step(const Launch& l, const GemmItem* items_dev, const SplitItem* sitems_dev,
                              const SliceBlock* blocks_dev, const SplitStep& step, const SplitBuffers& B,
                              int slices, const double2* Abuf, int64_t sA, const double2* Bbuf, int64_t sB,
-                             bool ready, int np, cudaStream_t st);
+                             bool ready, const SplitCopy& copy, int np, cudaStream_t st);
 cudaError_t split_mma_step(const Launch& l, int step_index, const GemmItem* items_dev,
                            const SplitItem* sitems_dev, const GemmTile* stiles_dev, const SplitStep& step,
                            const SplitBuffers& B, int slices, double2* Cbuf, int64_t sC, int np, int* status,

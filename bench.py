@@ -341,18 +341,34 @@ def _kernel_totals(prof):
 
 # DRAM bytes per launch of the dominant kernel (dram__bytes_read.sum + dram__bytes_write.sum,
 # averaged over its launches in one sweep) for a workload with default options, from a single-pass
-# ncu capture of the same kernel build; an entry is removed whenever the kernel changes.  The 3D
-# metallic lattice's entry: every split-GEMM launch of one full-size 8-point chunk (six slices),
+# ncu capture.  The 3D metallic lattice's entry is from the kernel before its slices took the shared
+# [Re | Im | -Im] format (B operands a quarter smaller now), so it bounds today's traffic from above:
+# every split-GEMM launch of one full-size 8-point chunk (six slices),
 # scaled to the sweep's mix of chunks (17 six-slice points, 144 five-slice poles, 21 chunks) in
 # proportion to points x slices.
 TRAFFIC_PER_LAUNCH = {("C5", "split", "gemm_split"): 3.52e9}
 TRAFFIC_SOURCE = {("C5", "split", "gemm_split"):
                   "ncu dram__bytes_read.sum + dram__bytes_write.sum of all 356 split-GEMM launches of "
                   "one 8-point six-slice chunk (4.31 GB per launch), scaled to the sweep's chunk mix; "
-                  "algorithmic bytes are ~1.5 GB per launch (operands re-read 2.4x)"}
+                  "algorithmic bytes were ~1.5 GB per launch (operands re-read 2.4x); taken before B slices "
+                  "shrank by a quarter"}
 
 
-def _roofline(prof, steps, peaks, fp64_peak, traffic_key=None):
+def _alu_peak(torch, multiply_adds):
+    """Rate of the FP64-accurate complex products on the CUDA cores, in TFLOP/s at 6 flops per product:
+    `multiply_adds` 32 x 32 + 64-bit integer multiply-adds each, 64 lanes per clock and SM at the maximum SM
+    clock (59 lanes measured in long independent chains)."""
+    import subprocess
+    try:
+        mhz = float(subprocess.run(["nvidia-smi", "--query-gpu=clocks.max.sm", "--format=csv,noheader,nounits"],
+                                   capture_output=True, text=True, timeout=20).stdout.split()[0])
+    except (OSError, ValueError, IndexError, subprocess.SubprocessError):
+        mhz = 2070.0
+    sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
+    return 6.0 * 64.0 / multiply_adds * sms * mhz * 1e6 / 1e12
+
+
+def _roofline(prof, steps, peaks, alu_peak, traffic_key=None):
     kern = _kernel_totals(prof)
     dname, d = max(kern.items(), key=lambda kv: kv[1]["ms"])
     total = sum(v["ms"] for v in kern.values())
@@ -364,19 +380,22 @@ def _roofline(prof, steps, peaks, fp64_peak, traffic_key=None):
                             "inside a long step)",
              "fp64_equivalent_tflops": d["flops"] / (d["ms"] * 1e-3) / 1e12}
     elif dname in ("gemm_f64", "diaginv"):
-        peak = fp64_peak
+        peak = alu_peak
         rate8 = d["flops"] / (d["ms"] * 1e-3) / 1e12
         r = {"bound": "alu", "unit": "TFLOP/s", "peak": peak,
-             "peak_source": "of measured (ndsi_fp64_peak in this run: DFMA chains on every SM)"}
+             "peak_source": "nine 32-bit integer multiply-adds per complex product (fixed-point products, "
+                            "FP64 sums) at 64 lanes per clock and SM and the maximum SM clock; the DFMA rate "
+                            "is fp64_peak_tflops_measured"}
         if dname == "gemm_f64":
             # the kernel's algorithm is the three-multiplication complex product: 3 real
-            # multiply-adds (6 flops) per complex multiply-add; the conventional count is 8
+            # multiply-adds (6 flops, three integer multiply-adds each) per complex multiply-add; the
+            # conventional count is 8
             achieved = 0.75 * rate8
             r.update(flop_count="6 per complex multiply-add (three-multiplication product, as executed)",
                      achieved_8flop_count=rate8, frac_8flop_count=rate8 / peak)
         else:
-            achieved = rate8
-            r["flop_count"] = "8 nb^3 per pivot block"
+            achieved = 0.75 * rate8
+            r["flop_count"] = "6 nb^3 per diagonal block (symmetry halves what is executed)"
     else:
         peak = peaks.get("hbm_gbs", 6792.7)
         achieved = d["bytes"] / (d["ms"] * 1e-3) / 1e9
@@ -494,7 +513,7 @@ def _release(torch):
     torch.cuda.empty_cache()
 
 
-def _other_leg(nd, torch, args, system, H, S, kT, M, stream, flush, prec_code, fp64_peak, ms_main,
+def _other_leg(nd, torch, args, system, H, S, kT, M, stream, flush, prec_code, ms_main,
                rho_main, ne_main):
     """The other precision on the same workload.  Every pole costs the same, so a large system's
     FP64 path is timed on a stated subset of the poles and compared per contour point; the two
@@ -515,7 +534,7 @@ def _other_leg(nd, torch, args, system, H, S, kT, M, stream, flush, prec_code, f
     w2, k2 = (max(args.warmup, 3), args.steps) if Mo == M else (1, 1)
     t2, prof2, _ = _measure(nd, torch, plan2, step2, k2, w2, stream, flush, 1)
     ms2 = sum(t2) / len(t2)
-    rl2, kk2 = _roofline(prof2, 1, _peaks(), fp64_peak)
+    rl2, kk2 = _roofline(prof2, 1, _peaks(), _alu_peak(torch, 9))
     per_point_main = ms_main / (M + 1)
     per_point_other = ms2 / (Mo + 1)
     split_pp, fp64_pp = ((per_point_other, per_point_main) if oprec == "split" else
@@ -657,7 +676,7 @@ def run_ndsi(args):
     del plan, step, e2e_step              # the headline plan's workspace goes back to the device
     if not args.no_other and rank == 0:
         other, fp64_ms_full = _other_leg(nd, torch, args, system, H, S, kT, M, stream, flush, prec_code,
-                                         fp64_peak, ms_step * world if world > 1 else ms_step, rho_main,
+                                         ms_step * world if world > 1 else ms_step, rho_main,
                                          ne_main)
     if rank != 0:
         if world > 1:
@@ -665,7 +684,7 @@ def run_ndsi(args):
         return 0
     default_opts = not (args.poles or args.outer or args.block or args.slices or args.bands or args.leaf
                         or args.far_ratio)
-    roofline, kern = _roofline(prof, len(prof_times), _peaks(), fp64_peak,
+    roofline, kern = _roofline(prof, len(prof_times), _peaks(), _alu_peak(torch, 9),
                                (args.config, args.precision) if default_opts else None)
     launches = sum(v["launches"] for v in kern.values())
     parity = None if args.no_parity else _parity(args, system, rho_main, kT, M, stored,
@@ -852,7 +871,7 @@ def run_batched(args, nd, torch, dist, rank, world, local, prec_code):
             checked.append({"system": i, "n": sy.n, "columns": cols})
         parity = {"max_abs_err_rho": err, "checked": checked,
                   "tolerance": 1e-10 if args.precision == "fp64" else 1e-9}
-    roofline, kern = _roofline(prof, args.steps, _peaks(), nd.ndsi_fp64_peak())
+    roofline, kern = _roofline(prof, args.steps, _peaks(), _alu_peak(torch, 9))
     line = {"metric": METRIC, "value": M * ntot / (ms * 1e-3), "unit": UNIT, "n_gpus": world,
             "steps": args.steps, "warmup": max(args.warmup, 3), "ms_per_step": ms,
             "higher_is_better": True, "scaling": "strong", "vs_baseline": None,
@@ -997,7 +1016,7 @@ def run_eigen(args):
     H = torch.as_tensor(system.H, device="cuda")
     S = torch.as_tensor(system.S, device="cuda")
     xi, n_states, block, eta = MU, 8, 12, 1e-3
-    fp64_peak = nd.ndsi_fp64_peak()
+    alu_peak = _alu_peak(torch, 12)
     nd.ndsi_eigenstates(plan, H, S, xi, n_states, eta=eta, block=block)          # warm
     t0 = time.perf_counter()
     eps, C, res, iters = nd.ndsi_eigenstates(plan, H, S, xi, n_states, eta=eta, block=block)
@@ -1037,13 +1056,11 @@ def run_eigen(args):
             "solve": {"rhs": k, "ms": ms_solve, "algorithmic_bytes": alg_bytes,
                       "gbs": alg_bytes / ms_solve / 1e6, "hbm_frac": alg_bytes / ms_solve / 1e6 / peak,
                       "roofline": {"bound": "alu", "unit": "TFLOP/s",
-                                   "achieved": 0.75 * alg_flops / ms_solve / 1e9, "peak": fp64_peak,
-                                   "frac": 0.75 * alg_flops / ms_solve / 1e9 / fp64_peak,
-                                   "flop_count": "6 per complex term (the three-multiplication form "
-                                                 "as executed; 8 in the conventional count)",
-                                   "peak_source": "of measured (ndsi_fp64_peak in this run); the "
-                                                  "solve is FP64-bound (each 16-byte factor element "
-                                                  "feeds 3 real FMAs per right-hand side)"}}}
+                                   "achieved": 0.75 * alg_flops / ms_solve / 1e9, "peak": alu_peak,
+                                   "frac": 0.75 * alg_flops / ms_solve / 1e9 / alu_peak,
+                                   "flop_count": "6 per complex term (8 in the conventional count)",
+                                   "peak_source": "twelve 32-bit integer multiply-adds per complex term at "
+                                                  "64 lanes per clock and SM and the maximum SM clock"}}}
     if system.n <= 4096 and not args.no_cpu:
         from oracle.eigen import eigenstates_near
         Hd, Sd = system.dense()

@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
+#include <type_traits>
 
 #include "fixed_point.cuh"
 #include "kernels.cuh"
@@ -34,7 +35,7 @@ __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_doub
 // (lanes = rows, 8 warps x 4 columns) and several poles, which share the tile's indices: the chain
 // tile -> node -> children -> index maps takes as long as the loads themselves.  A thread's eight loads
 // are in flight together, and FP64 additions (16 clocks of an SM per warp) are left out where one
-// child contributes.  80 poles of a cubic lattice of 16^3 atoms x 4 orbitals: 15.8 -> 12.1 ms, 5.2 TB/s.
+// child contributes.  80 poles of a cubic lattice of 16^3 atoms x 4 orbitals: 15.8 -> 10.8 ms, 5.8 TB/s.
 __global__ void __launch_bounds__(256) k_assemble(const NodeDev* __restrict__ nodes,
                                                   const NodeTile* __restrict__ tiles, int64_t first,
                                                   const int32_t* __restrict__ inv_map,
@@ -63,26 +64,33 @@ __global__ void __launch_bounds__(256) k_assemble(const NodeDev* __restrict__ no
             src[c][u] = has ? ch[c].front_off + ch[c].s + ia[c] + (static_cast<int64_t>(ch[c].s) + ibs[c][q]) * ch[c].f : -1;
         }
     const int64_t dst = nd.front_off + a + static_cast<int64_t>(t.j0 + ty) * f;
-    for (int pole = blockIdx.y; pole < np; pole += gridDim.y) {
-        double2* Fp = F + pole * stride;
-        double2 v[2][kCols];
+    auto run = [&](auto adds) {
+        for (int pole = blockIdx.y; pole < np; pole += gridDim.y) {
+            double2* Fp = F + pole * stride;
+            double2 v[2][kCols];
 #pragma unroll
-        for (int c = 0; c < 2; ++c)
+            for (int c = 0; c < 2; ++c)
+#pragma unroll
+                for (int u = 0; u < kCols; ++u) {
+                    v[c][u] = make_double2(0.0, 0.0);
+                    if (src[c][u] >= 0) v[c][u] = Fp[src[c][u]];
+                }
 #pragma unroll
             for (int u = 0; u < kCols; ++u) {
-                v[c][u] = make_double2(0.0, 0.0);
-                if (src[c][u] >= 0) v[c][u] = Fp[src[c][u]];
+                const bool one = src[0][u] >= 0, both = one && src[1][u] >= 0;
+                double2 o = make_double2(one ? v[0][u].x : v[1][u].x, one ? v[0][u].y : v[1][u].y);
+                if (decltype(adds)::value && both) o = cadd(v[0][u], v[1][u]);
+                const int b = t.j0 + ty + 8 * u;
+                if (b <= a && a < f) Fp[dst + static_cast<int64_t>(8 * u) * f] = o;
             }
-#pragma unroll
-        for (int u = 0; u < kCols; ++u) {
-            const bool one = src[0][u] >= 0, both = one && src[1][u] >= 0;
-            double2 o = make_double2(one ? v[0][u].x : v[1][u].x, one ? v[0][u].y : v[1][u].y);
-            if (__any_sync(0xffffffffu, both))
-                if (both) o = cadd(v[0][u], v[1][u]);
-            const int b = t.j0 + ty + 8 * u;
-            if (b <= a && a < f) Fp[dst + static_cast<int64_t>(8 * u) * f] = o;
         }
-    }
+    };
+    // two loops: an addition that no lane of a warp needs would still take its 64 clocks
+    bool both = false;
+#pragma unroll
+    for (int u = 0; u < kCols; ++u) both |= src[0][u] >= 0 && src[1][u] >= 0;
+    if (__any_sync(0xffffffffu, both)) run(std::true_type{});
+    else run(std::false_type{});
 }
 
 // Exponents of the basis scaling (launch_basis_scale): f_i from the exponent of S_ii, one thread per

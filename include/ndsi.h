@@ -42,11 +42,16 @@ extern "C" {
 #define NDSI_ERR_UNSUPPORTED  6   /* feature not available on this device or build */
 
 /* Arithmetic of the dense contractions (separator Schur updates and selected-inverse
- * products).  Diagonal blocks take the pivots in FP64 and their products in the same
- * fixed point, and the residue sum is FP64, in both. */
-#define NDSI_PREC_FP64   0   /* FP64 operands on the CUDA cores: products exact in 55-bit fixed point per
-                                operand row and 64 inner indices (integer multiply-adds), summed
-                                in FP64 */
+ * products).  In both, the basis functions are first brought to a common scale by powers of two
+ * (from S_ii, and from the size of the rows of H where on-site energies or couplings differ
+ * widely), diagonal blocks take their pivots in FP64 and their products in the fixed point of the
+ * FP64 mode, and the residue sum is FP64. */
+#define NDSI_PREC_FP64   0   /* FP64 operands on the CUDA cores.  Products are formed with integer
+                                multiply-adds in 55-bit fixed point relative to the largest element of
+                                an operand row over 64 inner indices (the product of the two low
+                                digits is dropped) and summed in FP64: errors are those of FP64
+                                products relative to the row and column maxima of the scaled
+                                matrices, not relative to every single element */
 #define NDSI_PREC_SPLIT  1   /* FP64 emulated by BF16 slices on the tcgen05 tensor cores */
 
 typedef struct ndsi_plan ndsi_plan;

@@ -27,6 +27,10 @@ int upload_tables(ndsi_plan* h) {
         void** dst;
     };
     DevTables& T = h->T;
+    std::vector<int64_t> diag(static_cast<size_t>(P.n));
+    for (int64_t i = 0; i < P.n; ++i)
+        diag[i] = std::lower_bound(P.col.begin() + P.rowptr[i], P.col.begin() + P.rowptr[i + 1], static_cast<int32_t>(i)) -
+                  P.col.begin();
     std::vector<Part> parts = {
         {P.nodes.data(), bytes_of(P.nodes), reinterpret_cast<void**>(&T.nodes)},
         {P.asm_map.data(), bytes_of(P.asm_map), reinterpret_cast<void**>(&T.asm_map)},
@@ -40,6 +44,7 @@ int upload_tables(ndsi_plan* h) {
         {P.diag_items.data(), bytes_of(P.diag_items), reinterpret_cast<void**>(&T.diag_items)},
         {P.node_tiles.data(), bytes_of(P.node_tiles), reinterpret_cast<void**>(&T.node_tiles)},
         {P.entry_sys.data(), bytes_of(P.entry_sys), reinterpret_cast<void**>(&T.entry_sys)},
+        {diag.data(), bytes_of(diag), reinterpret_cast<void**>(&T.diag)},
         {P.rowptr.data(), bytes_of(P.rowptr), reinterpret_cast<void**>(&T.rowptr)},
         {P.col.data(), bytes_of(P.col), reinterpret_cast<void**>(&T.col)},
         {nullptr, sizeof(int) * 4, reinterpret_cast<void**>(&T.status)},
@@ -102,9 +107,15 @@ int alloc_workspace(Workspace& W, const Plan& P, int32_t np) {
     W.scr_stride = P.scr_total;
     const size_t front_bytes = sizeof(double2) * static_cast<size_t>(W.front_stride) * np;
     NDSI_CK(cudaMalloc(&W.fronts, front_bytes + scale_bytes(P)));
-    W.scale_any = reinterpret_cast<int*>(reinterpret_cast<char*>(W.fronts) + front_bytes);
-    W.scale_f = reinterpret_cast<int16_t*>(W.scale_any + 64);
-    W.scale_pair = W.scale_f + P.n;
+    ScaleTables& t = W.scale;
+    t.any = reinterpret_cast<int*>(reinterpret_cast<char*>(W.fronts) + front_bytes);
+    t.stat = reinterpret_cast<ScaleStat*>(t.any + 64);
+    t.g[0] = reinterpret_cast<int*>(t.stat + P.n_systems);
+    t.g[1] = t.g[0] + P.n;
+    t.norm = reinterpret_cast<int16_t*>(t.g[1] + P.n);
+    t.ez = t.norm + P.n;
+    t.f = t.ez + P.n;
+    t.pair = t.f + P.n;
     NDSI_CK(cudaMalloc(&W.scr, sizeof(double2) * static_cast<size_t>(W.scr_stride) * np));
     W.np_cap = np;
     return NDSI_OK;
@@ -687,7 +698,7 @@ int ndsi_factor_poles(ndsi_plan* h, const double* H, const double* S, const doub
     }
     const double *Hd, *Sd;
     rc = device_inputs(h, H, S, &Hd, &Sd, st);
-    if (!rc && launch_basis_scale(h->P, h->T, Sd, f->W, st) != cudaSuccess)
+    if (!rc && launch_basis_scale(h->P, h->T, Hd, Sd, f->zd, 0, n_poles, f->W, st) != cudaSuccess)
         rc = fail(NDSI_ERR_CUDA, "ndsi_factor_poles: basis scaling launch failed");
     if (!rc) rc = run_phase(h, f->W, f->SB, 0, Hd, Sd, f->zd, 0, n_poles, st);
     if (rc) {
@@ -1004,7 +1015,7 @@ int sweep(ndsi_plan* h, const double* Hd, const double* Sd, int32_t nq, int32_t 
           const std::vector<int>& part_off, double* rho_d, double* ne_d, double* e_d, cudaStream_t st) {
     int rc;
     const int32_t ns = h->P.n_systems;
-    NDSI_CK(launch_basis_scale(h->P, h->T, Sd, h->W, st));
+    NDSI_CK(launch_basis_scale(h->P, h->T, Hd, Sd, h->zw, nq, nq, h->W, st));
     for (int32_t q0 = 0; q0 < nq;) {
         const bool far = q0 >= n_near;
         const int32_t np = std::min(chunk, (far ? nq : n_near) - q0);

@@ -140,7 +140,7 @@ int dos_sweep_systems(ndsi_plan* h, const double* Hd, const double* Sd, const do
         h->dos_part_cap = part_need;
     }
     NDSI_CK(cudaMemcpyAsync(h->dos_z, z.data(), sizeof(double2) * npts, cudaMemcpyHostToDevice, st));
-    NDSI_CK(launch_basis_scale(h->P, h->T, Sd, h->W, st));
+    NDSI_CK(launch_basis_scale(h->P, h->T, Hd, Sd, h->dos_z, nE, nE, h->W, st));
     for (int q0 = 0; q0 < nE; q0 += chunk) {
         const int np = std::min(chunk, nE - q0);
         rc = run_phase(h, h->W, h->SB, 0, Hd, Sd, h->dos_z + q0, nE, np, st);
@@ -148,7 +148,7 @@ int dos_sweep_systems(ndsi_plan* h, const double* Hd, const double* Sd, const do
         if (rc) return rc;
         for (int32_t sy = 0; sy < ns; ++sy) {
             const int64_t k0 = h->P.sys_nnz_first[sy], k1 = h->P.sys_nnz_first[sy + 1];
-            NDSI_CK(launch_point_traces_range(h->T.out_map + k0, h->W.scale_pair + k0, k1 - k0, h->W.fronts, h->W.front_stride, np, Sd + k0,
+            NDSI_CK(launch_point_traces_range(h->T.out_map + k0, h->W.scale.pair + k0, k1 - k0, h->W.fronts, h->W.front_stride, np, Sd + k0,
                                               h->dos_part, h->dos_tr + static_cast<int64_t>(sy) * nE + q0, st));
         }
     }

@@ -22,9 +22,9 @@ int ensure_solve_tables(ndsi_plan* h) {
 // Row exponents the solves with W's factors need (NULL for a normalised basis, where all are 0).
 int solve_scale(const Workspace& W, const int16_t** f, cudaStream_t st) {
     int any = 0;
-    NDSI_CK(cudaMemcpyAsync(&any, W.scale_any, sizeof(int), cudaMemcpyDeviceToHost, st));
+    NDSI_CK(cudaMemcpyAsync(&any, W.scale.any, sizeof(int), cudaMemcpyDeviceToHost, st));
     NDSI_CK(cudaStreamSynchronize(st));
-    *f = any ? W.scale_f : nullptr;
+    *f = any ? W.scale.f : nullptr;
     return NDSI_OK;
 }
 
@@ -73,7 +73,7 @@ int ndsi_factors_solve(ndsi_factors* f, int32_t pole, const double* Y, int32_t k
         f->scaled = sf ? 1 : 0;
     }
     NDSI_CK(launch_solve(h->P, h->ST, f->W.fronts + static_cast<int64_t>(pole) * f->W.front_stride, yw, xd, k,
-                         f->scaled ? f->W.scale_f : nullptr, st));
+                         f->scaled ? f->W.scale.f : nullptr, st));
     if (!x_dev) NDSI_CK(cudaMemcpyAsync(X_out, xd, bytes, cudaMemcpyDeviceToHost, st));
     NDSI_CK(cudaStreamSynchronize(st));
     return NDSI_OK;
@@ -105,7 +105,7 @@ int ndsi_eigenstates(ndsi_plan* h, const double* H, const double* S, double xi, 
     if (!h->point_z) NDSI_CK(cudaMalloc(&h->point_z, sizeof(double2)));
     const double2 z = make_double2(xi, eta);
     NDSI_CK(cudaMemcpyAsync(h->point_z, &z, sizeof(double2), cudaMemcpyHostToDevice, st));
-    NDSI_CK(launch_basis_scale(h->P, h->T, Sd, h->W, st));
+    NDSI_CK(launch_basis_scale(h->P, h->T, Hd, Sd, h->point_z, 1, 1, h->W, st));
     rc = run_phase(h, h->W, h->SB, 0, Hd, Sd, h->point_z, 1, 1, st);
     const int16_t* sf = nullptr;
     if (!rc) rc = solve_scale(h->W, &sf, st);

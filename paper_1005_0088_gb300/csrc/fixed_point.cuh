@@ -9,17 +9,20 @@ namespace ndsi {
 
 // Fixed-point products.  GB300 issues one warp-wide FP64 instruction per SM every 16-19 clocks (1.7-2
 // lanes a clock; 64 clocks per sub-partition) but 59 lanes a clock of 32 x 32 + 64-bit integer
-// multiply-adds (both measured), so products of complex matrices are formed in 57-bit fixed point:
-// over at most 32 inner indices every row of op(A) and column of op(B) is scaled by a power of two
-// and cut to x = (h 2^29 + l) 2^(E - 57), |h| <= 2^28, -2^28 <= l < 2^28.  Twelve integer
-// multiply-adds per complex product accumulate the h h and h l + l h sums exactly in 64 bits
-// (|sum| <= 2^62 and 2^63 over 32 terms; l l, below 2^-57 of the row times column maximum, is
-// dropped), and the sum is rounded once to FP64.  The error of an output is about 2^-57 of (row
-// maximum) x (column maximum) per term plus that one rounding, against one FP64 rounding per term
-// and accumulator of a DFMA loop.  The basis functions are brought to a common scale beforehand
-// (launch_basis_scale), so that a row's maximum speaks for the row.
-// Rows or columns holding an infinity or NaN give NaN.
-constexpr int kFixK = 32;          // inner indices per exact integer sum
+// multiply-adds (both measured), so products of complex matrices are formed in fixed point: over a
+// chunk of inner indices every row of op(A) and column of op(B) is scaled by a power of two and cut to
+// two integer digits, x = (h 2^LB + l) 2^(E - 2 LB + 1), and integer multiply-adds sum h h and h l + l h
+// exactly in 64 bits; l l is dropped, and the sum is rounded once to FP64.  Two forms:
+//  * the GEMMs and the diagonal blocks: LB = 28 (55 bits), chunks of at most 64 indices, three real
+//    products per complex one (Fix3Sum, below);
+//  * the solves: LB = 29 (57 bits), chunks of 16, four real products (FixSum): |h| <= 2^28 and
+//    -2^28 <= l < 2^28, so that over kFixK = 32 terms the sums stay within 2^62 (h h) and 2^63.
+// The error of an output is about 2^-(2 LB - 1) of (row maximum) x (column maximum) per term and one
+// rounding per chunk, against one FP64 rounding of every term in a DFMA loop: the bits of elements far below
+// their row's maximum are lost.  The basis functions are therefore brought to a common scale beforehand
+// (launch_basis_scale), so that a row's maximum speaks for the row; elements below 2^-(2 LB - 1) of it and
+// subnormal ones count as zero.  Rows or columns holding an infinity or NaN give NaN.
+constexpr int kFixK = 32;          // inner indices the four-product sums (FixSum) are exact over
 constexpr int kFixNonFinite = 1 << 20;  // row exponent of a row holding an infinity or NaN
 
 // Digits of x at row exponent field `emax` (x == 0 or its exponent field <= emax), LB bits in the low one:

@@ -72,7 +72,9 @@ typedef struct {
     int32_t split_slices;        /* BF16 slices per operand in split mode, 4..7; 0 (default) = 6 */
     int32_t block;               /* FP64 pivot block size, 16/32/64 (0 = default 16) */
     double m0_radius;            /* R of the zeroth-moment point Z = iR (default 1e7) */
-    int64_t max_workspace_bytes; /* device workspace cap; poles are chunked to fit (0 = auto) */
+    int64_t max_workspace_bytes; /* device workspace cap; poles are chunked to fit (0 = auto).  The basis
+                                    scaling tables (2 bytes per pattern entry, 14 per basis function)
+                                    count when poles are chunked; they alone fail no call */
     int32_t outer_block;         /* diagonal-block size of the two-level factorisation of A_J: the
                                     block's own LDL^T and inverse run in FP64 pivot blocks, the
                                     panel, trailing update and inverse assembly outside it are the

@@ -321,6 +321,14 @@ int64_t workspace_cap(const ndsi_plan* h) {
     return static_cast<int64_t>(0.85 * static_cast<double>(have));
 }
 
+int chunk_points(const ndsi_plan* h, int32_t points, int32_t* chunk) {
+    const int64_t per_pole = bytes_per_pole(h), cap = workspace_cap(h);
+    if (cap < per_pole) return NDSI_ERR_OOM;
+    const int64_t fit = (cap - static_cast<int64_t>(scale_bytes(h->P))) / per_pole;
+    *chunk = static_cast<int32_t>(std::min<int64_t>(points, std::max<int64_t>(1, fit)));
+    return NDSI_OK;
+}
+
 }  // namespace ndsi
 
 namespace ndsi {
@@ -926,10 +934,8 @@ int density_impl(ndsi_plan* h, const double* Hd, const double* Sd, const double*
         for (int32_t p = pf; p < pe; ++p) put_pole(q++, p);
     }
     // chunk the points to the workspace cap
-    const int64_t per_pole = bytes_per_pole(h);
-    int64_t cap = workspace_cap(h);
-    int32_t chunk = static_cast<int32_t>(std::min<int64_t>(nq, std::max<int64_t>(1, cap / per_pole)));
-    if (cap < per_pole) return fail(NDSI_ERR_OOM, "ndsi_density: one pole does not fit the workspace cap");
+    int32_t chunk = 0;
+    if (chunk_points(h, nq, &chunk)) return fail(NDSI_ERR_OOM, "ndsi_density: one pole does not fit the workspace cap");
     rc = alloc_workspace(h->W, h->P, chunk);
     if (rc) return rc;
     if (h->P.opt.precision == NDSI_PREC_SPLIT) NDSI_CK(split_alloc(h->SB, h->SP.steps, h->P.opt.split_slices, chunk));

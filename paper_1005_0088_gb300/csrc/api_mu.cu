@@ -113,10 +113,8 @@ int dos_sweep_systems(ndsi_plan* h, const double* Hd, const double* Sd, const do
     std::vector<double2> z(npts);
     for (int32_t sy = 0; sy < ns; ++sy)
         for (int k = 0; k < nE; ++k) z[static_cast<size_t>(sy) * nE + k] = make_double2(E[static_cast<size_t>(sy) * nE + k], eta[sy]);
-    const int64_t per_pole = bytes_per_pole(h);
-    const int64_t cap = workspace_cap(h);
-    if (cap < per_pole) return fail(NDSI_ERR_OOM, "ndsi_dos: one point does not fit the workspace cap");
-    const int32_t chunk = static_cast<int32_t>(std::min<int64_t>(nE, std::max<int64_t>(1, cap / per_pole)));
+    int32_t chunk = 0;
+    if (chunk_points(h, nE, &chunk)) return fail(NDSI_ERR_OOM, "ndsi_dos: one point does not fit the workspace cap");
     int rc = alloc_workspace(h->W, h->P, std::max<int32_t>(chunk, h->W.np_cap));
     if (rc) return rc;
     if (h->P.opt.precision == NDSI_PREC_SPLIT)

@@ -151,6 +151,9 @@ int alloc_workspace(Workspace& W, const Plan& P, int32_t np);
 void free_workspace(Workspace& W);
 int64_t bytes_per_pole(const ndsi_plan* h);
 int64_t workspace_cap(const ndsi_plan* h);
+// Points per chunk of a sweep over `points`: as many as fit the workspace cap beside the scaling tables, at least
+// one; NDSI_ERR_OOM when one point alone does not fit.
+int chunk_points(const ndsi_plan* h, int32_t points, int32_t* chunk);
 int ensure_stage(ndsi_plan* h, int64_t doubles);
 // H, S on the device (host inputs are staged); the device status word after a sweep.
 int device_inputs(ndsi_plan* h, const double* H, const double* S, const double** Hd, const double** Sd,

@@ -543,7 +543,8 @@ int ndsi_mlp_init(float* params, uint64_t seed, void* stream);
 /* Y[s] = network(X[s, :]) for s < n; X device float[n*32], Y device float[n]. */
 int ndsi_mlp_forward(const float* params, const float* X, int32_t n, float* Y, void* stream);
 /* grad (device float[NDSI_MLP_PARAMS]) and loss (device float, may be NULL) of the mean squared
- * error (1/n) sum_s (network(X_s) - T_s)^2.  Synchronises the stream. */
+ * error (1/n) sum_s (network(X_s) - T_s)^2.  Synchronises the stream.  Takes at most 16 MB of device
+ * memory during the call, as ndsi_mlp_train does, whatever n is. */
 int ndsi_mlp_grad(const float* params, const float* X, const float* T, int32_t n, float* grad,
                   float* loss, void* stream);
 /* `steps` full-batch Adam steps (beta1 0.9, beta2 0.999) on the mean squared error; final loss

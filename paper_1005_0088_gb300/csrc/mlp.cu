@@ -3,6 +3,7 @@
 // (Sec. II.C.3); this network only proposes the starting bracket for that search.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <string>
@@ -19,7 +20,11 @@ constexpr int kNW1 = kHid * kIn, kNB1 = kHid, kNW2 = kHid * kHid, kNB2 = kHid, k
 constexpr int kOffW1 = 0, kOffB1 = kOffW1 + kNW1, kOffW2 = kOffB1 + kNB1, kOffB2 = kOffW2 + kNW2,
               kOffW3 = kOffB2 + kNB2, kOffB3 = kOffW3 + kNW3, kNParams = kOffB3 + kNB3;
 static_assert(kNParams == NDSI_MLP_PARAMS, "parameter layout");
-constexpr int kBatchBlock = 16;  // samples per CTA in the gradient kernel: 125 CTAs for 2000 samples
+constexpr int kBatchBlock = 16;  // samples a CTA of the gradient kernel takes at a time: 125 CTAs for 2000 samples
+// CTAs of the gradient kernel at most (four fit an SM): each then takes several groups of samples, so that the
+// partial gradients stay within 15 MB for any number of samples.
+constexpr int kGradBlocks = 4 * 152;
+inline int grad_blocks(int n) { return std::min(n / kBatchBlock + (n % kBatchBlock != 0), kGradBlocks); }
 
 // SplitMix64 (Steele, Lea, Flood 2014) as a counter-based generator.
 __host__ __device__ inline uint64_t splitmix64(uint64_t x) {
@@ -124,12 +129,12 @@ __global__ void __launch_bounds__(128) k_mlp_forward(const float* __restrict__ p
     Y[s] = y;
 }
 
-// Mean-squared-error gradient of a block of up to 16 samples, written as one partial gradient per block
+// Mean-squared-error gradient of groups of up to 16 samples, summed over a block's groups, one partial gradient per block
 // (summed in a fixed order by k_mlp_reduce, so the result is deterministic).  The work is small
 // (37 kflop per sample) and latency decides: all 256 threads share every layer (an output neuron and
 // four samples each), activations lie neuron-major with the samples as float4, weights row-padded
-// against bank conflicts.  2000 samples: 140 -> 15 us per training step with k_mlp_reduce (one thread
-// per sample over 64-sample blocks left 120 SMs idle and ran 37 kflop serially).
+// against bank conflicts.  A call of 25 training steps on 2000 samples, with k_mlp_reduce: 3.46 -> 0.69 ms (one
+// thread per sample over 64-sample blocks left 120 SMs idle and ran 37 kflop serially).
 struct MlpShared {
     float w1[kHid][kIn + 1], w2[kHid][kHid + 1], w3[kHid], b1[kHid], b2[kHid], b3;
     float4 x[kIn][kBatchBlock / 4], h1[kHid][kBatchBlock / 4 + 1], h2[kHid][kBatchBlock / 4 + 1];
@@ -151,13 +156,14 @@ __device__ __forceinline__ float4 dtanh4(const float4& a, const float4& h) {
     return make_float4(a.x * (1.f - h.x * h.x), a.y * (1.f - h.y * h.y), a.z * (1.f - h.z * h.z), a.w * (1.f - h.w * h.w));
 }
 
+// ONE: a single group per block (a loop that may come again costs 7% of a call of 25 steps).
+template <bool ONE>
 __global__ void __launch_bounds__(256) k_mlp_grad(const float* __restrict__ params, const float* __restrict__ X,
                                                   const float* __restrict__ T, int n, float* __restrict__ partial,
                                                   float* __restrict__ loss_partial) {
     extern __shared__ float4 mlp_smem[];
     MlpShared& m = *reinterpret_cast<MlpShared*>(mlp_smem);
     const int tid = threadIdx.x;
-    const int s0 = blockIdx.x * kBatchBlock, nb = min(kBatchBlock, n - s0);
     for (int i = tid; i < kNW1; i += 256) m.w1[i / kIn][i % kIn] = params[kOffW1 + i];
     for (int i = tid; i < kNW2; i += 256) m.w2[i / kHid][i % kHid] = params[kOffW2 + i];
     if (tid < kHid) {
@@ -166,59 +172,61 @@ __global__ void __launch_bounds__(256) k_mlp_grad(const float* __restrict__ para
         m.w3[tid] = params[kOffW3 + tid];
     }
     if (tid == 0) m.b3 = params[kOffB3];
-    for (int i = tid; i < kBatchBlock * kIn; i += 256) {
-        const int b = i / kIn, k = i % kIn;
-        reinterpret_cast<float*>(m.x[k])[b] = b < nb ? X[static_cast<int64_t>(s0 + b) * kIn + k] : 0.f;
-    }
-    __syncthreads();
-    const int j = tid % kHid, g = tid / kHid;  // a neuron and a group of four samples
-    {
-        float4 a = make_float4(m.b1[j], m.b1[j], m.b1[j], m.b1[j]);
-#pragma unroll 8
-        for (int i = 0; i < kIn; ++i) fma4(a, m.w1[j][i], m.x[i][g]);
-        m.h1[j][g] = tanh4(a);
-    }
-    __syncthreads();
-    {
-        float4 a = make_float4(m.b2[j], m.b2[j], m.b2[j], m.b2[j]);
-#pragma unroll 8
-        for (int i = 0; i < kHid; ++i) fma4(a, m.w2[j][i], m.h1[i][g]);
-        m.h2[j][g] = tanh4(a);
-    }
-    __syncthreads();
-    {
-        // output and its error: sixteen threads per sample, four neurons each
-        const int b = tid / 16, q = tid % 16;
-        float a = 0.f;
-#pragma unroll
-        for (int u = 0; u < kHid / 16; ++u) a = fmaf(m.w3[q + 16 * u], reinterpret_cast<const float*>(m.h2[q + 16 * u])[b], a);
-#pragma unroll
-        for (int o = 8; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-        if (q == 0) {
-            const float e = b < nb ? a + m.b3 - T[s0 + b] : 0.f;
-            m.dy[b] = 2.f * e / static_cast<float>(n);
-            m.l[b] = e * e / static_cast<float>(n);
-        }
-    }
-    __syncthreads();
-    {
-        const float4 dy = *reinterpret_cast<const float4*>(&m.dy[4 * g]);
-        const float w = m.w3[j];
-        m.dz2[j][g] = dtanh4(make_float4(dy.x * w, dy.y * w, dy.z * w, dy.w * w), m.h2[j][g]);
-    }
-    __syncthreads();
-    {
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 8
-        for (int i = 0; i < kHid; ++i) fma4(a, m.w2[i][j], m.dz2[i][g]);
-        m.dz1[j][g] = dtanh4(a, m.h1[j][g]);
-    }
-    __syncthreads();
+    const int j = tid % kHid, g = tid / kHid;    // a neuron and a group of four samples
+    const int r0 = tid / 16, c0 = tid % 16;      // dW2 = dz2^T h1 in 4 x 4 register tiles, dW1 = dz1^T x in 4 x 2
+    float dw2[4][4] = {}, dw1[4][2] = {}, db1 = 0.f, db2 = 0.f, dw3 = 0.f, db3 = 0.f, lsum = 0.f;
+    const int groups = n / kBatchBlock + (n % kBatchBlock != 0);
     float* out = partial + static_cast<int64_t>(blockIdx.x) * kNParams;
-    // dW2 = dz2^T h1 in 4 x 4 register tiles, dW1 = dz1^T x in 4 x 2
-    const int r0 = tid / 16, c0 = tid % 16;
-    {
-        float a[4][4] = {};
+    for (int grp = blockIdx.x;; grp += gridDim.x) {
+        const bool last = ONE || groups - grp <= static_cast<int>(gridDim.x);
+        const int s0 = grp * kBatchBlock, nb = min(kBatchBlock, n - s0);
+        for (int i = tid; i < kBatchBlock * kIn; i += 256) {
+            const int b = i / kIn, k = i % kIn;
+            reinterpret_cast<float*>(m.x[k])[b] = b < nb ? X[static_cast<int64_t>(s0 + b) * kIn + k] : 0.f;
+        }
+        __syncthreads();
+        {
+            float4 a = make_float4(m.b1[j], m.b1[j], m.b1[j], m.b1[j]);
+#pragma unroll 8
+            for (int i = 0; i < kIn; ++i) fma4(a, m.w1[j][i], m.x[i][g]);
+            m.h1[j][g] = tanh4(a);
+        }
+        __syncthreads();
+        {
+            float4 a = make_float4(m.b2[j], m.b2[j], m.b2[j], m.b2[j]);
+#pragma unroll 8
+            for (int i = 0; i < kHid; ++i) fma4(a, m.w2[j][i], m.h1[i][g]);
+            m.h2[j][g] = tanh4(a);
+        }
+        __syncthreads();
+        {
+            // output and its error: sixteen threads per sample, four neurons each
+            const int b = tid / 16, q = tid % 16;
+            float a = 0.f;
+#pragma unroll
+            for (int u = 0; u < kHid / 16; ++u) a = fmaf(m.w3[q + 16 * u], reinterpret_cast<const float*>(m.h2[q + 16 * u])[b], a);
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+            if (q == 0) {
+                const float e = b < nb ? a + m.b3 - T[s0 + b] : 0.f;
+                m.dy[b] = 2.f * e / static_cast<float>(n);
+                m.l[b] = e * e / static_cast<float>(n);
+            }
+        }
+        __syncthreads();
+        {
+            const float4 dy = *reinterpret_cast<const float4*>(&m.dy[4 * g]);
+            const float w = m.w3[j];
+            m.dz2[j][g] = dtanh4(make_float4(dy.x * w, dy.y * w, dy.z * w, dy.w * w), m.h2[j][g]);
+        }
+        __syncthreads();
+        {
+            float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+            for (int i = 0; i < kHid; ++i) fma4(a, m.w2[i][j], m.dz2[i][g]);
+            m.dz1[j][g] = dtanh4(a, m.h1[j][g]);
+        }
+        __syncthreads();
 #pragma unroll
         for (int b = 0; b < kBatchBlock / 4; ++b) {
             float4 u[4], v[4];
@@ -230,51 +238,56 @@ __global__ void __launch_bounds__(256) k_mlp_grad(const float* __restrict__ para
 #pragma unroll
             for (int p = 0; p < 4; ++p)
 #pragma unroll
-                for (int q = 0; q < 4; ++q) a[p][q] = dot4(u[p], v[q], a[p][q]);
+                for (int q = 0; q < 4; ++q) dw2[p][q] = dot4(u[p], v[q], dw2[p][q]);
+        }
+        if (last) {
+#pragma unroll
+            for (int p = 0; p < 4; ++p)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) out[kOffW2 + (r0 + 16 * p) * kHid + c0 + 16 * q] = dw2[p][q];
         }
 #pragma unroll
-        for (int p = 0; p < 4; ++p)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) out[kOffW2 + (r0 + 16 * p) * kHid + c0 + 16 * q] = a[p][q];
-    }
-    {
-        float a[4][2] = {};
-#pragma unroll
         for (int b = 0; b < kBatchBlock / 4; ++b) {
-            float4 v[2] = {m.x[c0][b], m.x[c0 + 16][b]};
+            const float4 v[2] = {m.x[c0][b], m.x[c0 + 16][b]};
 #pragma unroll
             for (int p = 0; p < 4; ++p) {
                 const float4 u = m.dz1[r0 + 16 * p][b];
 #pragma unroll
-                for (int q = 0; q < 2; ++q) a[p][q] = dot4(u, v[q], a[p][q]);
+                for (int q = 0; q < 2; ++q) dw1[p][q] = dot4(u, v[q], dw1[p][q]);
             }
         }
+        if (last) {
 #pragma unroll
-        for (int p = 0; p < 4; ++p)
+            for (int p = 0; p < 4; ++p)
 #pragma unroll
-            for (int q = 0; q < 2; ++q) out[kOffW1 + (r0 + 16 * p) * kIn + c0 + 16 * q] = a[p][q];
-    }
-    if (tid < kHid) {  // db1, db2, dW3
-        float a = 0.f, c = 0.f, w = 0.f;
-#pragma unroll
-        for (int b = 0; b < kBatchBlock / 4; ++b) {
-            const float4 one = make_float4(1.f, 1.f, 1.f, 1.f);
-            a = dot4(m.dz1[tid][b], one, a);
-            c = dot4(m.dz2[tid][b], one, c);
-            w = dot4(*reinterpret_cast<const float4*>(&m.dy[4 * b]), m.h2[tid][b], w);
+                for (int q = 0; q < 2; ++q) out[kOffW1 + (r0 + 16 * p) * kIn + c0 + 16 * q] = dw1[p][q];
         }
-        out[kOffB1 + tid] = a;
-        out[kOffB2 + tid] = c;
-        out[kOffW3 + tid] = w;
-    }
-    if (tid == 0) {  // db3 and the block's loss
-        float a = 0.f, l = 0.f;
-        for (int b = 0; b < kBatchBlock; ++b) {
-            a += m.dy[b];
-            l += m.l[b];
+        if (tid < kHid) {
+#pragma unroll
+            for (int b = 0; b < kBatchBlock / 4; ++b) {
+                const float4 one = make_float4(1.f, 1.f, 1.f, 1.f);
+                db1 = dot4(m.dz1[tid][b], one, db1);
+                db2 = dot4(m.dz2[tid][b], one, db2);
+                dw3 = dot4(*reinterpret_cast<const float4*>(&m.dy[4 * b]), m.h2[tid][b], dw3);
+            }
         }
-        out[kOffB3] = a;
-        loss_partial[blockIdx.x] = l;
+        if (tid == 0) {
+            for (int b = 0; b < kBatchBlock; ++b) {
+                db3 += m.dy[b];
+                lsum += m.l[b];
+            }
+        }
+        if (last) break;
+        __syncthreads();  // the next group's samples take the space
+    }
+    if (tid < kHid) {
+        out[kOffB1 + tid] = db1;
+        out[kOffB2 + tid] = db2;
+        out[kOffW3 + tid] = dw3;
+    }
+    if (tid == 0) {
+        out[kOffB3] = db3;
+        loss_partial[blockIdx.x] = lsum;
     }
 }
 
@@ -357,8 +370,9 @@ size_t grad_smem() { return sizeof(MlpShared); }
 
 int grad_launch(const float* params, const float* X, const float* T, int n, float* partial, float* lossp,
                 float* grad, float* loss, const AdamStep& adam, cudaStream_t st) {
-    const int nblk = (n + kBatchBlock - 1) / kBatchBlock;
-    k_mlp_grad<<<nblk, 256, grad_smem(), st>>>(params, X, T, n, partial, lossp);
+    const int nblk = grad_blocks(n);
+    const bool one = n <= kGradBlocks * kBatchBlock;
+    (one ? k_mlp_grad<true> : k_mlp_grad<false>)<<<nblk, 256, grad_smem(), st>>>(params, X, T, n, partial, lossp);
     MLP_CK(cudaGetLastError());
     k_mlp_reduce<<<(kNParams + 31) / 32, 256, 0, st>>>(partial, nblk, grad, lossp, loss, adam);
     MLP_CK(cudaGetLastError());
@@ -439,12 +453,12 @@ int ndsi_mlp_grad(const float* params, const float* X, const float* T, int32_t n
         return mfail(NDSI_ERR_INVALID, "ndsi_mlp_grad: device arrays and n >= 1 required");
     static bool attr = false;
     if (!attr) {
-        MLP_CK(cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    static_cast<int>(grad_smem())));
+        for (auto f : {&k_mlp_grad<true>, &k_mlp_grad<false>})
+            MLP_CK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(grad_smem())));
         attr = true;
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int nblk = (n + kBatchBlock - 1) / kBatchBlock;
+    const int nblk = grad_blocks(n);
     float *partial = nullptr, *lossp = nullptr;
     MLP_CK(cudaMalloc(&partial, sizeof(float) * (static_cast<size_t>(nblk) * kNParams + nblk)));
     lossp = partial + static_cast<size_t>(nblk) * kNParams;
@@ -462,12 +476,12 @@ int ndsi_mlp_train(float* params, const float* X, const float* T, int32_t n, int
         return mfail(NDSI_ERR_INVALID, "ndsi_mlp_train: device arrays, n >= 1, steps >= 1, lr > 0 required");
     static bool attr = false;
     if (!attr) {
-        MLP_CK(cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    static_cast<int>(grad_smem())));
+        for (auto f : {&k_mlp_grad<true>, &k_mlp_grad<false>})
+            MLP_CK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(grad_smem())));
         attr = true;
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int nblk = (n + kBatchBlock - 1) / kBatchBlock;
+    const int nblk = grad_blocks(n);
     float* work = nullptr;
     const size_t nwork = static_cast<size_t>(nblk) * kNParams + nblk + 2 * kNParams + 1;
     MLP_CK(cudaMalloc(&work, sizeof(float) * nwork));

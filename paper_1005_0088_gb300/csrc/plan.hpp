@@ -160,6 +160,10 @@ int merge_plans(std::vector<Plan>& parts, Plan& merged, std::string& err);
 
 // Bounds and write-overlap check of every schedule table (plan_check.cpp).
 int check_plan(const Plan& P, std::string& err);
+// May the copies of the launch `copy` be done before the GEMM launch `gemm` that they follow?  Their
+// destinations must meet no result of the GEMM and no operand that it still reads from the fronts (a `shared`
+// operand is read from its slices).
+bool copy_may_precede(const Plan& P, const Launch& gemm, const Launch& copy, bool a_shared, bool b_shared);
 
 // Chemical-potential search over caller-supplied evaluations (mu_search.cpp).
 int mu_search(ndsi_mu_eval_fn eval, ndsi_mu_dos_fn dos, void* ctx, double elo, double ehi, double kT,

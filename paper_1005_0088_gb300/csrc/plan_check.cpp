@@ -125,6 +125,32 @@ struct Checker {
         return false;
     }
 
+    // See copy_may_precede (plan.hpp).
+    bool copy_precedes(const Launch& g, const Launch& c, bool a_shared, bool b_shared) {
+        std::vector<Region> dst(c.count);
+        for (int64_t i = 0; i < c.count; ++i) {
+            const CopyItem& x = P.copy_items[c.first + i];
+            if (!region(BUF_FRONT, x.dst_off, x.ldd, x.rows, x.cols, dst[i], "copy destination")) return false;
+        }
+        Writes W;
+        if (!build_writes(dst, W, "copy")) return false;
+        for (int64_t i = 0; i < g.count; ++i) {
+            const GemmItem& x = P.gemm_items[g.first + i];
+            int64_t ar, ac, br, bc;
+            extent(g.opA, x.M, x.K, ar, ac);
+            extent(g.opB, x.K, x.N, br, bc);
+            Region A, B, C;
+            if (!region(g.bufA, x.a_off, x.lda, ar, ac, A, "GEMM operand A") ||
+                !region(g.bufB, x.b_off, x.ldb, br, bc, B, "GEMM operand B") ||
+                !region(g.bufC, x.c_off, x.ldc, x.M, x.N, C, "GEMM result"))
+                return false;
+            if ((g.bufC == BUF_FRONT && meets(W, C, -1)) || (!a_shared && g.bufA == BUF_FRONT && meets(W, A, -1)) ||
+                (!b_shared && g.bufB == BUF_FRONT && meets(W, B, -1)))
+                return fail("a copy's destination meets what the GEMM before it reads or writes");
+        }
+        return true;
+    }
+
     bool run() {
         // node records and index maps
         for (int32_t j = 0; j < P.n_nodes; ++j) {
@@ -233,6 +259,11 @@ struct Checker {
 };
 
 }  // namespace
+
+bool copy_may_precede(const Plan& P, const Launch& gemm, const Launch& copy, bool a_shared, bool b_shared) {
+    std::string err;
+    return Checker(P, err).copy_precedes(gemm, copy, a_shared, b_shared);
+}
 
 int check_plan(const Plan& P, std::string& err) {
     Checker c(P, err);

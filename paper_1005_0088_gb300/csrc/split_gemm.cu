@@ -222,6 +222,9 @@ void build_split_schedule(const Plan& P, int slices, const std::vector<int8_t>& 
                             : c.src_off != g.b_off || c.lds != g.ldb || c.rows != g.K || c.cols != g.N)
                     st.fuse_copy = 0;
             }
+            // the copy then comes before the GEMM: its destination may be the shared operand, whose slices are
+            // made, but nothing else that the step reads or writes
+            if (!copy_may_precede(P, l, P.launches[li + 1], takes_a, takes_b)) st.fuse_copy = 0;
         }
         auto cols = [&](int32_t parts) { return (std::max(64, parts * kmax) + 63) / 64 * 64; };
         st.A.Kcols = takes_a ? steps.back().B.Kcols : cols(st.A.parts);

@@ -306,17 +306,18 @@ int ndsi_profile_enable(ndsi_plan* plan, int32_t enable);
 /* Autotuner for split-precision plans: times every GEMM step of one density sweep at (mu, kT,
  * n_poles) on H, S (device or host) both on the tensor cores (slicing + emulated-FP64 GEMM) and
  * on the FP64 CUDA cores, with CUDA events per launch after an untimed warm-up of each, and keeps
- * the faster path per step for all later calls on the plan.  Both paths meet the split-mode
- * tolerance, so only speed changes.  Small steps (few tiles, short inner dimension) usually go
- * to the CUDA cores, separator-sized ones to the tensor cores.  A step whose tensor-core time is
- * below the least time the CUDA cores could need for it (their integer multiply-add rate) is
- * decided without an FP64 run, so on large systems
- * the FP64 sweeps time only the small steps.  A plan with the default accumulators (one per
- * slice scale) then times every tensor-core step once more with five accumulator bands (48
+ * the faster path per step for all later calls on the plan; steps that share the slices of an
+ * operand are decided in pairs, since the second one's time depends on the first one's path.  Both
+ * paths meet the split-mode tolerance, so only speed changes.  Small steps (few tiles, short inner
+ * dimension) usually go to the CUDA cores, separator-sized ones to the tensor cores.  A step whose
+ * tensor-core time is below the least time the CUDA cores could need for it (their integer
+ * multiply-add rate) is decided without an FP64 run, so on large systems the FP64 sweeps time only
+ * the small steps.  A plan with the default accumulators (one per slice scale) then times every
+ * tensor-core step, on the paths chosen, once more with five accumulator bands (48
  * complex columns per tile instead of 40, within the same tolerance) and keeps the faster tile per
  * step (NDSI_EXPORT_TILE_SHAPES lists the result); factors made before the call can no longer be
  * inverted by ndsi_selinv.  Counts of the steps left on each path in
- * *n_split_out / *n_fp64_out (either may be NULL).  Runs four to six sweeps; the profiler counters are
+ * *n_split_out / *n_fp64_out (either may be NULL).  Runs four to seven sweeps; the profiler counters are
  * unchanged and any captured graph is dropped.  FP64 plans: no-op (all steps
  * counted as FP64).  Errors: NDSI_ERR_INVALID for bad arguments or a batched plan; as
  * ndsi_density otherwise. */

@@ -1,5 +1,6 @@
 // C-ABI entry points: plan life cycle, pole-batched factor / selected inversion / density.
 #include "handle.hpp"
+#include "tune.hpp"
 
 namespace ndsi {
 
@@ -1180,8 +1181,9 @@ int ndsi_autotune(ndsi_plan* h, const double* H, const double* S, double mu, dou
     double* ne_d = h->stage + 3 * h->P.nnz;
     // Per-launch event timing of one sweep with every eligible GEMM on the tensor cores and one
     // with every eligible GEMM on the FP64 CUDA cores (each after an untimed warm-up sweep); each
-    // launch then keeps the faster of the two.  Both choices meet the split tolerance, so the
-    // result only changes speed.  The profiler's own counters are left as they were.
+    // step, or pair of steps that share slices, then keeps the fastest of the paths (choose_paths), after
+    // one more sweep where that is a pair not yet timed together.  All choices meet the split tolerance, so
+    // the result only changes speed.  The profiler's own counters are left as they were.
     // A step whose tensor-core time is already below the least time the FP64 path could take (nine
     // integer multiply-adds per complex product at 64 lanes per clock and SM, k_gemm_f64's bound) is
     // decided without running it on the CUDA cores: only the other steps are timed there.
@@ -1213,11 +1215,26 @@ int ndsi_autotune(ndsi_plan* h, const double* H, const double* S, double mu, dou
         h->prof.per_launch = pass == 0 ? nullptr : &t_fp64;
         rc = density_impl(h, Hd, Sd, &mu, &kT, n_poles, rho_d, ne_d, st);
     }
+    std::vector<TuneStep> steps;
+    for (size_t li = 0; li < nl; ++li) {
+        if (!split_eligible(h->P.launches[li])) continue;
+        const SplitStep& step = h->SP.steps[h->SP.step_of_launch[li]];
+        const bool copied = li + 1 < nl && h->P.launches[li + 1].kind == L_COPY;
+        steps.push_back(TuneStep{li, step.A.shared != 0 || step.B.shared != 0, copied ? static_cast<int64_t>(li + 1) : -1,
+                                 decided[li] != 0});
+    }
+    std::vector<char> use(nl, 1);
+    std::vector<double> t_b0;
+    if (!rc && choose_paths(steps, t_split, t_fp64, nullptr, nullptr, use, t_b0)) {
+        std::vector<double> t_mixed(nl, 0.0);
+        const std::vector<char> mixed_use = use;
+        h->SP.use_split = mixed_use;
+        h->prof.per_launch = &t_mixed;
+        rc = density_impl(h, Hd, Sd, &mu, &kT, n_poles, rho_d, ne_d, st);
+        if (!rc) choose_paths(steps, t_split, t_fp64, &t_mixed, &mixed_use, use, t_b0);
+    }
     h->prof.per_launch = nullptr;
-    for (size_t li = 0; li < nl; ++li)
-        h->SP.use_split[li] = !rc && split_eligible(h->P.launches[li])
-                                  ? (decided[li] || t_split[li] <= t_fp64[li] ? 1 : 0)
-                                  : 1;
+    h->SP.use_split = rc ? std::vector<char>(nl, 1) : use;
     // Tile shape of each tensor-core step: one accumulator per scale (40 complex columns per
     // tile, the plan default) or five accumulator bands (48 columns, a floor near 2^-43 of the
     // result, well inside the split tolerance).  The wider tile carries more multiply-adds per
@@ -1237,7 +1254,7 @@ int ndsi_autotune(ndsi_plan* h, const double* H, const double* S, double mu, dou
         }
         h->prof.per_launch = nullptr;
         for (size_t li = 0; li < nl; ++li)
-            h->SP.bands[li] = (!rc && h->SP.bands[li] == 5 && t_b5[li] < t_split[li]) ? 5 : 0;
+            h->SP.bands[li] = (!rc && h->SP.bands[li] == 5 && t_b5[li] < t_b0[li]) ? 5 : 0;
         const int rc2 = rebuild_split(h);
         if (!rc) rc = rc2;
     }

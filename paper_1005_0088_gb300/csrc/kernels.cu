@@ -26,6 +26,11 @@ __device__ __forceinline__ double scale2(double x, int e) {
     if (e == 0) return x;
     return e >= -1022 && e <= 1023 ? x * __hiloint2double((1023 + e) << 20, 0) : ldexp(x, e);
 }
+// |p|^2 of a pivot that cannot be inverted: zero or non-finite (decided on its bits, off the FP64 pipe).
+__device__ __forceinline__ bool bad_pivot(double den) {
+    const uint32_t hi = static_cast<uint32_t>(__double2hiint(den)) & 0x7FFFFFFFu;
+    return hi >= 0x7FF00000u || (hi | static_cast<uint32_t>(__double2loint(den))) == 0;
+}
 __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 
 // ---------------------------------------------------------------------------------------------
@@ -393,7 +398,7 @@ __global__ void __launch_bounds__(32) k_diaginv_sweep(const DiagItem* __restrict
         __syncwarp();
         const double2 p = cs[t];
         const double den = p.x * p.x + p.y * p.y;
-        bad |= (static_cast<uint32_t>(__double2hiint(den)) >> 20) - 1u >= 0x7FEu;  // zero, subnormal, non-finite
+        bad |= bad_pivot(den);
         const double rden = 1.0 / den;
         const double2 ip = make_double2(p.x * rden, -p.y * rden), nip = make_double2(-ip.x, -ip.y);
         if (lane < N) ds[lane] = cmul(cs[lane], ip);
@@ -543,8 +548,7 @@ __global__ void __launch_bounds__(512) k_diaginv_block(const DiagItem* __restric
                 const double2 p = X[tri(q, q)];
                 const double2 c = idx == q ? make_double2(1.0, 0.0) : X[tri(idx, q)];
                 const double den = p.x * p.x + p.y * p.y;
-                // zero, subnormal or non-finite: decided on the exponent field, off the FP64 pipe
-                bad |= (static_cast<uint32_t>(__double2hiint(den)) >> 20) - 1u >= 0x7FEu;
+                bad |= bad_pivot(den);
                 const double u = im ? c.y : c.x, v = im ? -c.x : c.y;
                 const double d = fma(u, p.x, v * p.y) * pivot_rcp(den);
                 reinterpret_cast<double*>(ds + idx)[im] = d;

@@ -19,7 +19,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CU_SOURCES = ["kernels.cu", "api.cu", "api_mu.cu", "api_solve.cu", "static_scratch.cu", "split_gemm.cu", "mlp.cu",
               "solve.cu", "peak.cu"]
 CPP_SOURCES = ["analyze.cpp", "mu_search.cpp", "plan_check.cpp", "small_eig.cpp", "tune.cpp"]
-HEADERS = ["plan.hpp", "kernels.cuh", "fixed_point.cuh", "split_gemm.cuh", "solve.cuh", "handle.hpp", "small_eig.hpp",
+HEADERS = ["plan.hpp", "kernels.cuh", "fixed_point.cuh", "pivot.cuh", "split_gemm.cuh", "solve.cuh", "handle.hpp", "small_eig.hpp",
            "tune.hpp"]
 
 

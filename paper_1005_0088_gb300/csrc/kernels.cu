@@ -97,7 +97,8 @@ __global__ void __launch_bounds__(256) k_assemble(const NodeDev* __restrict__ no
 // ---------------------------------------------------------------------------------------------
 // Basis scaling (launch_basis_scale): four passes over the pattern, one warp per row, bound by the
 // latency of a row's dependent loads (its columns, then their diagonals or scales), so four entries of a lane
-// are in flight together: 12 us a sweep for 320,000 entries instead of 25 one at a time, 2 us for 12,000.
+// are in flight together (12 us a sweep for 320,000 entries instead of 25 one at a time).  Against scales from S_ii
+// alone a sweep takes 6 us longer for 12,000 entries (0.96 -> 0.97 ms) and 16 us for 260,000 (7.84 -> 7.85 ms).
 // Exponent of |x| (|x| < 2^e); zero, subnormal and non-finite
 // values do not take part.
 constexpr int kNoExpo = -4000;
@@ -449,7 +450,7 @@ __host__ __device__ constexpr size_t diag_block_smem(int tile) {
            sizeof(int) * 4 + sizeof(uint16_t) * nb8 * (nb8 + 1) / 2;                // counters, unit list
 }
 
-// Threads per block of up to `tile` columns: narrow blocks leave room for three CTAs (64 columns, 65 KB
+// Threads per block of up to `tile` columns: narrow blocks leave room for three CTAs (64 columns, 71 KB
 // each) or two (80 columns) on an SM, whose pivot inversions then overlap; a 128-column block fills
 // one SM's shared memory and uses 16 warps for its updates.
 constexpr int diag_block_threads(int tile) { return tile <= 64 ? 128 : tile <= 80 ? 256 : 512; }
@@ -666,8 +667,8 @@ __global__ void __launch_bounds__(512) k_diaginv_block(const DiagItem* __restric
                 }
             }
         };
-        // the next pivot block is updated first, in six 8 x 4 pieces over the warps, and one warp
-        // inverts it while the others update the rest
+        // the next pivot block is updated first, in six 8 x 4 pieces over the warps, and the first four
+        // warps invert it while the others update the rest
         const bool ahead = t + 1 < nt;
         if (ahead) {
             const int N0 = 2 * t + 2;
@@ -1161,11 +1162,6 @@ cudaError_t launch_point_traces_range(const int64_t* out_map, const int16_t* pai
         e = cudaGetLastError();
     }
     return e;
-}
-
-cudaError_t launch_point_traces(const Plan& P, const DevTables& T, const Workspace& W, int np, const double* S,
-                                double* partials, double* out, cudaStream_t st) {
-    return launch_point_traces_range(T.out_map, W.scale.pair, P.nnz, W.fronts, W.front_stride, np, S, partials, out, st);
 }
 
 cudaError_t launch_reduce(const double* partials, int nblocks, double* out, cudaStream_t st) {

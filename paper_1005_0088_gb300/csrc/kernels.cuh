@@ -114,15 +114,12 @@ cudaError_t launch_gershgorin(const DevTables& T, int64_t n, const double* H, co
                               unsigned long long* out, cudaStream_t st);
 double gershgorin_value(unsigned long long key);
 
-// Per point q of a chunk: out[q] = sum over the pattern of Im G_q(k) S_k = Im Tr(G(z_q) S) (the
-// density of states of Eq. 42 up to -2/pi).  partials: np x accumulate_blocks(nnz) doubles.
-// The same over one range of pattern entries (out_map and S offset to its first entry; F holds np
-// point slabs of `stride` complex elements): out[q] = sum_k Im F_q[out_map[k]] 2^pair[k] S[k].
+// Per point q of a chunk, over a range of pattern entries (out_map, pair and S offset to its first entry; F holds
+// np point slabs of `stride` complex elements): out[q] = sum_k Im F_q[out_map[k]] 2^pair[k] S[k], over a whole
+// system Im Tr(G(z_q) S) (the density of states of Eq. 42 up to -2/pi).  partials: np x accumulate_blocks(nnz) doubles.
 cudaError_t launch_point_traces_range(const int64_t* out_map, const int16_t* pair, int64_t nnz, const double2* F,
                                       int64_t stride, int np, const double* S, double* partials, double* out,
                                       cudaStream_t st);
-cudaError_t launch_point_traces(const Plan& P, const DevTables& T, const Workspace& W, int np,
-                                const double* S, double* partials, double* out, cudaStream_t st);
 
 // G_out[q*nnz + k] = G_q(k) for the np poles of the workspace.
 cudaError_t launch_gather_pattern(const Plan& P, const DevTables& T, const Workspace& W, int np,

@@ -341,17 +341,11 @@ def _kernel_totals(prof):
 
 # DRAM bytes per launch of the dominant kernel (dram__bytes_read.sum + dram__bytes_write.sum,
 # averaged over its launches in one sweep) for a workload with default options, from a single-pass
-# ncu capture.  The 3D metallic lattice's entry is from the kernel before its slices took the shared
-# [Re | Im | -Im] format (B operands a quarter smaller now), so it bounds today's traffic from above:
-# every split-GEMM launch of one full-size 8-point chunk (six slices),
-# scaled to the sweep's mix of chunks (17 six-slice points, 144 five-slice poles, 21 chunks) in
-# proportion to points x slices.
-TRAFFIC_PER_LAUNCH = {("C5", "split", "gemm_split"): 3.52e9}
+# ncu capture of the present kernel: a figure becomes None whenever the kernel, its operands' format or
+# its tile order changes.  The split GEMM has none since its tiles move in rings and its slices are shared.
+TRAFFIC_PER_LAUNCH = {("C5", "split", "gemm_split"): None}
 TRAFFIC_SOURCE = {("C5", "split", "gemm_split"):
-                  "ncu dram__bytes_read.sum + dram__bytes_write.sum of all 356 split-GEMM launches of "
-                  "one 8-point six-slice chunk (4.31 GB per launch), scaled to the sweep's chunk mix; "
-                  "algorithmic bytes were ~1.5 GB per launch (operands re-read 2.4x); taken before B slices "
-                  "shrank by a quarter"}
+                  "not measured: no ncu capture of the present kernel on this workload"}
 
 
 def _alu_peak(torch, multiply_adds):
@@ -395,14 +389,15 @@ def _roofline(prof, steps, peaks, alu_peak, traffic_key=None):
                      achieved_8flop_count=rate8, frac_8flop_count=rate8 / peak)
         else:
             achieved = 0.75 * rate8
-            r["flop_count"] = "6 nb^3 per diagonal block (symmetry halves what is executed)"
+            r["flop_count"] = ("6 per complex multiply-add of a block's LDL^T and inverse by 16-wide pivot blocks "
+                               "(3.1 nb^3 at 128 columns, 3.2 at 64, 3.5 at 40)")
     else:
         peak = peaks.get("hbm_gbs", 6792.7)
         achieved = d["bytes"] / (d["ms"] * 1e-3) / 1e9
         r = {"bound": "hbm", "unit": "GB/s", "peak": peak,
              "peak_source": "of measured (MEASURED_PEAKS.json hbm_gbs)"}
     traffic = TRAFFIC_PER_LAUNCH.get(traffic_key + (dname,)) if traffic_key else None
-    if traffic is not None:
+    if traffic_key and traffic_key + (dname,) in TRAFFIC_SOURCE:
         r["traffic_source"] = TRAFFIC_SOURCE[traffic_key + (dname,)]
     r.update({"kernel": dname, "achieved": achieved, "frac": achieved / peak, "traffic": traffic,
               "launches": d["launches"], "kernel_ms_per_step": d["ms"] / steps,

@@ -21,7 +21,9 @@
 //    of two and exact in FP32 (scales 0-3; the lower ones, 2^-32 and below, may round at 2^-24 of
 //    themselves).  The accumulators are read out into a per-element float-float (hi, lo) sum
 //    at the ends of chunks of 256: scales 2 and 3 after every chunk, scale 1 after every second, the
-//    others after every fourth, and all at the end of a tile (split_read_mask).  The optional tail
+//    others after every fourth, and all at the end of a tile (split_read_mask); fewer read-outs round the pair's
+//    low part less often (a host model's rms error against all scales every 256: 1.00 of it at five slices,
+//    0.5-1.0 at six, 0.2-0.6 at seven, K = 512 to 4096).  The optional tail
 //    variants keep t+u = 2 .. BANDS in their own accumulators and the rest in a shared tail, read out
 //    after every chunk, where the tensor core drops the low bits of the smaller products: BANDS = 5
 //    (NC = 48) gives a floor near 2^-43 of the result, BANDS = 4 (NC = 64) near 2^-38;
@@ -41,7 +43,8 @@
 // first and are given back after 2/7 of the block, the A digits one by one, so that every load has
 // most of a block's time (4000 clocks at six digits; a load from L2 takes 2100) to arrive.  What
 // bounds it now is shared memory: a block's products read 360 KB of operands and the loads write
-// 156 KB, 4000 clocks at 128 bytes each against 3360 of tensor work.  Of the rest, 6% is the wait for
+// 156 KB, 4000 clocks at 128 bytes each against 3360 of tensor work (M = 800, N = K = 4000: 6.89 -> 6.01 ms, tensor pipe
+// 57 -> 66% busy, shared memory 56% by operand reads and 23% by loads).  Of the rest, 6% is the wait for
 // read-outs (with all six accumulators read every chunk: 20%) and 15% late loads.  Measured against
 // the two-stage form: 3D metallic lattice T = G_RR L_RJ 1435 -> 1519 TFLOP/s issued, Schur update
 // 1131 -> 1284; 3D cubic lattice 803 -> 967 (Schur); blocks that end with each part (below) cost
